@@ -187,7 +187,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmx, const PrefillArgs p,
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) unsigned long long bars[3 * kMaxStages + 5];
   __shared__ unsigned tmem_base_s;
-  __shared__ int abort_s;
+  __shared__ int abort_s, go_s;
   volatile int* abort_flag = &abort_s;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -209,6 +209,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmx, const PrefillArgs p,
   const int first_tile = (int)blockIdx.x - slice * ntiles;
   const int my_tiles = first_tile < ntiles ? (ntiles - 1 - first_tile) / (int)gridDim.x + 1 : 0;
 
+  const bool go = tid == 64 && no_one_gave_up(p.status);   // on its way while the barriers are set up
   if (tid == 0) {
     abort_s = 0;
     for (int s = 0; s < stages; ++s) {
@@ -229,11 +230,12 @@ prefill_kernel(const __grid_constant__ CUtensorMap tmx, const PrefillArgs p,
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if (tid == 64) go_s = go;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned tmem_acc = tmem_base_s;
-  bool ok = *reinterpret_cast<volatile int32_t*>(p.status) == 0;   // an earlier CTA gave up: do no work
+  bool ok = go_s != 0;   // an earlier CTA gave up: do no work
   int issued = 0;   // k-block copies started (producer thread only), counted over all tiles
 
   if (warp == 0) {
@@ -568,7 +570,9 @@ __global__ void __launch_bounds__(256) expand_outliers_kernel(const int32_t* __r
 //                        shared-memory tile of 32 tokens x 128 features that one thread hands to a TMA store (whole
 //                        256-byte rows of y instead of 2 bytes per thread); both CTAs' epilogue warps tell the first
 //                        CTA when an accumulator is free again.
-// Every wait is bounded (see the fused kernel); the two CTAs leave together through a cluster barrier.
+// Every wait for another role is bounded (see the fused kernel), and the four epilogue warps, which meet at a named barrier
+// inside a tile, go by one verdict each time: the pair's at the start, theirs after every wait.  The two CTAs leave together
+// through a cluster barrier.
 constexpr int kPairThreads = 32 * 6;
 // TOK tokens per tile of a pair (UMMA N; 256, or 128 where that fills the pairs better), half of them loaded by each CTA
 template <int TOK> struct PairCfg {
@@ -587,6 +591,11 @@ __device__ __forceinline__ unsigned in_first_cta(unsigned addr) {
   unsigned r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
   return r;
+}
+__device__ __forceinline__ int load_cluster(unsigned cluster_addr) {
+  int v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+  return v;
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -660,7 +669,7 @@ pair_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUt
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) unsigned long long bars[2 * 8 + 5];
   __shared__ unsigned tmem_base_s;
-  __shared__ int abort_s;
+  __shared__ int abort_s, go_s;
   volatile int* abort_flag = &abort_s;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -715,12 +724,14 @@ pair_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUt
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  cluster_sync_all();   // both CTAs' barriers exist before either signals the other
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const unsigned tmem_acc = tmem_base_s;
   pdl_trigger();
   pdl_sync();   // the operands are written, and y may still be read, by the kernels before
-  bool ok = *reinterpret_cast<volatile int32_t*>(p.status) == 0;   // an earlier CTA gave up: do no work
+  if (tid == 0 && rank == 0) go_s = no_one_gave_up(p.status);
+  __syncwarp();
+  cluster_sync_all();   // both CTAs' barriers, and the pair's verdict, exist before either signals the other
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const unsigned tmem_acc = tmem_base_s;
+  bool ok = load_cluster(in_first_cta(smem_u32(&go_s))) != 0;   // an earlier CTA gave up: do no work, neither CTA of the pair
   int issued = 0;   // k-block copies started (producer thread only), counted over all tiles
 
   if (warp == 0) {

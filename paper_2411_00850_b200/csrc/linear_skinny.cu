@@ -104,7 +104,7 @@ skinny_kernel(const __grid_constant__ CUtensorMap tmc, const __grid_constant__ C
   float* xsum = reinterpret_cast<float*>(out_tiles + kSets * kOutTileBytes);     // [kXs][AS][TOK]
   __shared__ __align__(8) unsigned long long bars[2 * kStages + 2 * kSets + 4 + 4 + 2 * kXs + 1];
   __shared__ unsigned tmem_base_s;
-  __shared__ int abort_s;
+  __shared__ int abort_s, go_s;
   volatile int* abort_flag = &abort_s;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -134,6 +134,7 @@ skinny_kernel(const __grid_constant__ CUtensorMap tmc, const __grid_constant__ C
   auto tile_of = [&](int j) { return (int)(tile0 + (grp0 + (unsigned)j) / (unsigned)G); };
   auto grp_of = [&](int j) { return (int)((grp0 + (unsigned)j) % (unsigned)G); };
 
+  const bool go = tid == 64 && no_one_gave_up(p.status);   // on its way while the barriers are set up
   if (tid == 0) {
     abort_s = 0;
     for (int s = 0; s < kStages; ++s) {
@@ -167,6 +168,7 @@ skinny_kernel(const __grid_constant__ CUtensorMap tmc, const __grid_constant__ C
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if (tid == 64) go_s = go;
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -176,7 +178,7 @@ skinny_kernel(const __grid_constant__ CUtensorMap tmc, const __grid_constant__ C
   auto tm_d = [&](int d) { return tmem0 + (unsigned)(128 + d * TOK); };
   auto tm_o = [&](int o) { return tmem0 + (unsigned)(128 + 2 * TOK + o * TOK); };
   asm volatile("griddepcontrol.launch_dependents;");
-  bool ok = *reinterpret_cast<volatile int32_t*>(p.status) == 0;   // an earlier launch gave up: do no work
+  bool ok = go_s != 0;   // an earlier launch gave up: do no work
   int issued = 0;   // stages armed by the producer
 
   if (warp == kWarpProducer) {

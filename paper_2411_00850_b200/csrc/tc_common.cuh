@@ -52,6 +52,14 @@ static __device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned par
   return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, limit));
 }
 
+// True while no kernel has given up on the layer (later calls then do no work until the host has read the status).  Other
+// CTAs write the word while this one starts, so a CTA must go by ONE read of it: one thread reads, before a barrier of all
+// that share its verdict, and hands it round through shared memory.  Warps that each looked for themselves could start with
+// different verdicts, and one that skips its loop never comes to the barriers inside it.
+static __device__ __forceinline__ bool no_one_gave_up(const int32_t* status) {
+  return *reinterpret_cast<const volatile int32_t*>(status) == 0;
+}
+
 static __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* map, int c0, int c1, unsigned bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"

@@ -35,3 +35,29 @@ def test_zero_spin_limit_gives_up_cleanly_and_the_layer_stays_usable(N, K, M):
         assert gwq.gwq_device_status(P) == 0
         assert_linear_close(y, y_ref, bound)
     P.free()
+
+
+# Give-ups while other CTAs of the launch are still starting, many times over: one pair of CTAs after the other finds the
+# status word written between the reads of its warps.  More pairs than one round holds, K-slices of the last round, the
+# fused kernel in slices; then a call that finds the word set, which skips its work and leaves y alone.
+@pytest.mark.parametrize("N,K,M", [(600, 512, 2200), (4096, 512, 2400), (2816, 4096, 1000), (1024, 2048, 64)])
+def test_give_ups_of_a_whole_grid_end_every_time(N, K, M):
+    W, G = synth.make_weight_and_grad(N, K, 96)
+    P = quantize_on_gpu(W, G, 0.01, 4, 128)
+    bits16, _ = synth.make_activations(M, K, seed=96, dtype="f16")
+    x = x_tensor(bits16, "f16")
+    want = gwq.gwq_linear(P, x)
+    assert gwq.gwq_device_status(P) == 0
+    for _ in range(60):
+        gwq.gwq_set_wait_limit(P, 0)
+        gwq.gwq_linear(P, x)
+        gwq.gwq_set_wait_limit(P, -1)
+        assert gwq.gwq_device_status(P) == gwq.GWQ_ERR_TIMEOUT
+    gwq.gwq_set_wait_limit(P, 0)
+    gwq.gwq_linear(P, x)
+    gwq.gwq_set_wait_limit(P, -1)
+    gwq.gwq_linear(P, x)                                    # the word is set: no work, no wait
+    assert gwq.gwq_device_status(P) == gwq.GWQ_ERR_TIMEOUT
+    assert torch.equal(gwq.gwq_linear(P, x), want)
+    assert gwq.gwq_device_status(P) == 0
+    P.free()
