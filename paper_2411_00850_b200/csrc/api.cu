@@ -17,20 +17,20 @@ static bool wants_skinny(const gwq_packed* P, gwq_dtype xd, int M) {
          gwq_skinny_takes(P, xd, M);
 }
 
-static bool takes_few(const gwq_packed* P, int M) { return gwq_decode_ahead(P, M) || gwq_stream_takes(P, M); }
+static bool takes_few(const gwq_packed* P, gwq_dtype xd, int M) { return gwq_decode_ahead(P, xd, M) || gwq_stream_takes(P, M); }
 // Layers that read the same x, up to 32 tokens, in one launch: the kernel that each layer takes by itself.
 static gwq_status launch_few(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M, void* const* y,
                              gwq_dtype yd, cudaStream_t stream) {
-  const bool rows = gwq_decode_ahead(P[0], M);
+  const bool rows = gwq_decode_ahead(P[0], xd, M);
   for (int i = 1; i < count; ++i)
-    if (gwq_decode_ahead(P[i], M) != rows) return GWQ_ERR_UNSUPPORTED;
+    if (gwq_decode_ahead(P[i], xd, M) != rows) return GWQ_ERR_UNSUPPORTED;
   return rows ? gwq_launch_decode_multi(P, count, x, xd, M, y, yd, stream) : gwq_launch_stream(P, count, x, xd, M, y, yd, stream);
 }
 
 extern "C" size_t gwq_linear_workspace_bytes(const gwq_packed* P, gwq_dtype xd, int32_t M) {
   if (!P || P->tag != GWQ_TAG_PACKED || !P->priv || M <= 0) return 0;
   if (wants_skinny(P, xd, M)) return gwq_skinny_workspace_bytes(P, M);
-  if (M <= GWQ_DECODE_MAX_M && takes_few(P, M)) return 0;
+  if (M <= GWQ_DECODE_MAX_M && takes_few(P, xd, M)) return 0;
   return gwq_prefill_workspace_bytes(P, xd, M);
 }
 
@@ -120,8 +120,8 @@ static gwq_status linear_host(gwq_packed* P, const void* x_host, gwq_dtype xd, i
   // transposing pre-pass, or, where every CTA reads them, by a kernel that copies them first) and y is
   // written once, so that nothing is gained by the copy engine, whose two copies take longer than the product
   // (4096 x 11008 at 4 tokens: 47 -> 34 us).
-  const bool direct = M <= GWQ_DECODE_MAX_M && !wants_skinny(P, xd, M) && takes_few(P, M);
-  const bool copied = M == 1 || (direct && gwq_decode_ahead(P, M));
+  const bool direct = M <= GWQ_DECODE_MAX_M && !wants_skinny(P, xd, M) && takes_few(P, xd, M);
+  const bool copied = M == 1 || (direct && gwq_decode_ahead(P, xd, M));
   const void* x = direct && gwq_aligned16(x_host) ? device_view(x_host, xb) : nullptr;
   void* y = direct && yb <= kDirectMostBytes ? device_view(y_host, yb) : nullptr;
   if (!x || copied) GWQ_CUDA_TRY(grow(&pv->x_stage, &pv->x_stage_bytes, xb, stream));

@@ -85,7 +85,7 @@ gwq_status gwq_launch_simt(const gwq_packed* P, const void* x, gwq_dtype xd, int
                            gwq_dtype yd, cudaStream_t stream);
 gwq_status gwq_launch_decode_multi(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M,
                                    void* const* y, gwq_dtype yd, cudaStream_t stream);
-bool gwq_decode_ahead(const gwq_packed* P, int M);   // the kernel with a CTA per tile is the faster one for (P, M)
+bool gwq_decode_ahead(const gwq_packed* P, gwq_dtype xd, int M);   // the kernel with a CTA per tile is the faster one for (P, xd, M)
 gwq_status gwq_launch_prefill(const gwq_packed* P, const void* x, gwq_dtype xd, int M, void* y,
                               gwq_dtype yd, void* ws, size_t ws_bytes, cudaStream_t stream);
 size_t gwq_prefill_workspace_bytes(const gwq_packed* P, gwq_dtype xd, int M);

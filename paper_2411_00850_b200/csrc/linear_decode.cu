@@ -152,7 +152,7 @@ bool plan(const gwq_packed* const* P, int count, int M, Variant* v, int* cvcap) 
 // CTAs, and its lanes do less per code of one or four tokens; the streaming kernel's cost per code hardly grows up to eight
 // tokens, its activations are shared by all tiles of a CTA, and one wave of its CTAs covers any layer, unevenly where they
 // get between one tile and a little more than two.  Ratios are this kernel's time to the streaming one's.
-bool gwq_decode_ahead(const gwq_packed* P, int M) {
+bool gwq_decode_ahead(const gwq_packed* P, gwq_dtype xd, int M) {
   Variant v;
   int cvcap;
   if (!plan(&P, 1, M, &v, &cvcap)) return false;
@@ -161,6 +161,17 @@ bool gwq_decode_ahead(const gwq_packed* P, int M) {
   const long long weights = (long long)P->N * P->K;
   const bool g128 = P->group == 128, lone = tiles <= sms, uneven = tiles > 2 * sms && 2 * tiles <= 9 * sms;
   const bool fitting = 2 * tiles <= 9 * sms;   // up to four and a half tiles per SM
+  // bf16 activations: the streaming kernel then multiplies by q - z as this one does, one packed add per two codes more, and is
+  // ahead where its other savings outweigh that.  One token: groups of 128 0.81 to 0.95 (4 bits beyond ten tiles per SM 1.04, 2
+  // bits up to two 1.04 to 1.22), groups of 64 0.74 to 1.03 in between, 1.01 to 1.28 up to two tiles per SM, 0.99 to 1.08 beyond
+  // ten.  Five to eight tokens: groups of 128 0.71 to 1.0 (with x in a ring and two tiles per SM 1.0 to 1.04, 2 bits with a
+  // tile per SM 1.28 to 1.35); groups of 64 with 3 bits 0.77 to 1.0, with 4 bits up to four and a half tiles per SM 0.89 to
+  // 1.0, beyond 0.91 to 1.12.
+  if (xd == GWQ_BF16 && bits != 8 && P->group >= 64) {
+    if (M == 1) return (g128 && bits == 3) || (tiles <= 10 * sms && (tiles > 2 * sms || (g128 && bits == 4)));
+    if (M > 4 && M <= 8 && g128) return bits == 2 ? !lone : v.nbuf == 0 || tiles > 2 * sms;
+    if (M > 4 && M <= 8 && bits != 2) return bits == 3 || fitting;
+  }
   // 8 bits: 0.56 to 1.0.  3 bits: 0.78 on 6144 x 8192, 0.93 on 4096 x 4096 (with groups of 64 on uneven grids only).
   // Otherwise long rows of grids that leave the streaming kernel's last CTAs out: 0.88 on 3000 x 24064, 1.07 on 4736 x 8832.
   if (M == 1) {
