@@ -153,9 +153,10 @@ gwq_status gwq_pack(const uint16_t* W_f16, gwq_outliers* S, int32_t N, int32_t K
  *   always for layers with fewer 128-row tiles than the device has SMs) expands the weights once instead of
  *   once per token tile and contracts on pairs of CTAs (tcgen05 cta_group::2, tiles of 256 features x 256 tokens).
  *   Asynchronous on `stream`: the call only enqueues kernels.  It never allocates and never
- *   synchronises, so it may be captured into a CUDA graph from its first use.  Calls that share P
- *   must be enqueued on one stream (or otherwise ordered): with 9 to 32 tokens they share a small
- *   scratch buffer that gwq_pack created inside P.
+ *   synchronises, so it may be captured into a CUDA graph from its first use.  Calls that share P and have
+ *   9 to 32 tokens must be enqueued on one stream (or otherwise ordered): they share a small scratch buffer
+ *   that gwq_pack created inside P.  Calls of up to 8 tokens share nothing (where the kernel would need scratch, they
+ *   are served a few tokens at a time), nor do calls of gwq_linear_ws with a workspace of their own.
  *   A call that cannot do without scratch (bf16 activations on the tensor-core path need an fp16 copy of
  *   x) returns GWQ_ERR_WORKSPACE and does nothing: make it through gwq_linear_ws.  Calls that merely run
  *   faster with scratch take their slower kernel here.
@@ -164,7 +165,7 @@ gwq_status gwq_linear(const gwq_packed* P, const void* x, gwq_dtype x_dtype, int
                       gwq_dtype y_dtype, void* stream);
 
 /* gwq_linear with scratch memory supplied by the caller.  gwq_linear_workspace_bytes returns the bytes
- * the product (P, x_dtype, M) needs (0 when it needs none); `workspace` must be a device buffer of at
+ * the product (P, x_dtype, M) needs, or runs faster with (0 when it has no use for any); `workspace` must be a device buffer of at
  * least that size, 256-byte aligned, and must not be used by anything else until the kernels enqueued by
  * the call have finished (calls on one stream may share it).  Otherwise exactly gwq_linear.
  * Errors: as gwq_linear; WORKSPACE when workspace_bytes is too small or the buffer is misaligned.  */
@@ -178,15 +179,20 @@ gwq_status gwq_linear_ws(const gwq_packed* P, const void* x, gwq_dtype x_dtype, 
  * exactly the one gwq_linear computes, bit for bit.
  *   P: host array of `count` packed layers (1 <= count <= GWQ_MULTI_MAX) with the same K.
  *   x: device [M, K]; y: host array of `count` device pointers, y[i] is [M, P[i]->N], all of y_dtype.
- *   With M <= 32, one group size (64 or 128) and one bit width for all layers, the products run as ONE kernel
- *   launch wherever the streaming kernel takes that shape (layer 0 lends its scratch: do not overlap with
- *   another call that uses P[0]); otherwise the call is the same as `count` calls of gwq_linear in order
- *   (and like them returns GWQ_ERR_WORKSPACE where a product needs scratch: call gwq_linear_ws per layer
- *   then).  Asynchronous on `stream`; never allocates, never synchronises.
+ *   With M <= 32, one group size and one bit width for all layers, the products run as ONE kernel launch wherever
+ *   all layers take the same decode kernel by themselves (with 9 to 32 tokens layer 0 lends its scratch: do not overlap
+ *   with another such call that uses P[0]); otherwise the call is the same as `count` calls of gwq_linear in order
+ *   (and like them returns GWQ_ERR_WORKSPACE where a product needs scratch).  Asynchronous on `stream`; never
+ *   allocates, never synchronises.
+ * gwq_linear_multi_ws: with scratch memory supplied by the caller, as in gwq_linear_ws (each product is then exactly the one
+ *   gwq_linear_ws computes); gwq_linear_multi_workspace_bytes: its size.
  * Errors: INVALID_ARG (count, null entries, differing K, alignment), otherwise as gwq_linear.          */
 #define GWQ_MULTI_MAX 4
 gwq_status gwq_linear_multi(const gwq_packed* const* P, int32_t count, const void* x, gwq_dtype x_dtype,
                             int32_t M, void* const* y, gwq_dtype y_dtype, void* stream);
+size_t gwq_linear_multi_workspace_bytes(const gwq_packed* const* P, int32_t count, gwq_dtype x_dtype, int32_t M);
+gwq_status gwq_linear_multi_ws(const gwq_packed* const* P, int32_t count, const void* x, gwq_dtype x_dtype, int32_t M,
+                               void* const* y, gwq_dtype y_dtype, void* workspace, size_t workspace_bytes, void* stream);
 
 /* Mean of the gradients of `count` calibration samples (Section 4.3, "Effect on Number of Calibration":
  * the outliers are located on the gradient mean); the result feeds gwq_select_outliers.

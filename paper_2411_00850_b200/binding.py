@@ -28,7 +28,7 @@ STATUS_NAMES = {
     4: "GWQ_ERR_NONFINITE", 5: "GWQ_ERR_TIMEOUT", 6: "GWQ_ERR_CUDA", 7: "GWQ_ERR_WORKSPACE",
 }
 EXPORTS = ("gwq_select_outliers", "gwq_select_outliers_static", "gwq_outliers_rows", "gwq_pack", "gwq_linear", "gwq_linear_ws",
-           "gwq_linear_workspace_bytes", "gwq_linear_multi",
+           "gwq_linear_workspace_bytes", "gwq_linear_multi", "gwq_linear_multi_ws", "gwq_linear_multi_workspace_bytes",
            "gwq_gradient_mean", "gwq_quality", "gwq_linear_host", "gwq_linear_host_async", "gwq_device_status", "gwq_set_wait_limit", "gwq_free", "gwq_status_string")
 GWQ_MULTI_MAX = 4
 
@@ -86,6 +86,11 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
     lib.gwq_linear_multi.restype = C.c_int
     lib.gwq_linear_multi.argtypes = [C.POINTER(C.POINTER(gwq_packed)), C.c_int32, C.c_void_p, C.c_int, C.c_int32,
                                      C.POINTER(C.c_void_p), C.c_int, C.c_void_p]
+    lib.gwq_linear_multi_ws.restype = C.c_int
+    lib.gwq_linear_multi_ws.argtypes = [C.POINTER(C.POINTER(gwq_packed)), C.c_int32, C.c_void_p, C.c_int, C.c_int32,
+                                        C.POINTER(C.c_void_p), C.c_int, C.c_void_p, C.c_size_t, C.c_void_p]
+    lib.gwq_linear_multi_workspace_bytes.restype = C.c_size_t
+    lib.gwq_linear_multi_workspace_bytes.argtypes = [C.POINTER(C.POINTER(gwq_packed)), C.c_int32, C.c_int, C.c_int32]
     lib.gwq_gradient_mean.restype = C.c_int
     lib.gwq_gradient_mean.argtypes = [C.POINTER(C.c_void_p), C.c_int32, C.c_int64, C.c_void_p, C.c_void_p]
     lib.gwq_quality.restype = C.c_int
@@ -265,7 +270,8 @@ def gwq_linear(P: Packed, x: torch.Tensor, out_dtype: torch.dtype | None = None,
                out: torch.Tensor | None = None, workspace: torch.Tensor | None = None) -> torch.Tensor:
     """y = x (deq(Wq) + S)^T for x [M,K] fp16/bf16 on the GPU; asynchronous on the current stream.
     Where the product needs scratch memory (gwq_linear_workspace_bytes > 0) it is taken from `workspace`
-    (a CUDA uint8 tensor) or, by default, from a new torch tensor: the library itself never allocates here."""
+    (a CUDA uint8 tensor) or, by default, from a new torch tensor: the library itself never allocates here, and calls
+    on one layer share nothing."""
     return (_ext or _load_ext()).linear(P._addr, x, out_dtype, out, workspace)
 
 

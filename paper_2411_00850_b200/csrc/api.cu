@@ -18,19 +18,58 @@ static bool wants_skinny(const gwq_packed* P, gwq_dtype xd, int M) {
 }
 
 static bool takes_few(const gwq_packed* P, gwq_dtype xd, int M) { return gwq_decode_ahead(P, xd, M) || gwq_stream_takes(P, M); }
-// Layers that read the same x, up to 32 tokens, in one launch: the kernel that each layer takes by itself.
-static gwq_status launch_few(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M, void* const* y,
-                             gwq_dtype yd, cudaStream_t stream) {
-  const bool rows = gwq_decode_ahead(P[0], xd, M);
+bool gwq_takes_decode(const gwq_packed* P, gwq_dtype xd, int M) {
+  return M <= GWQ_DECODE_MAX_M && !wants_skinny(P, xd, M) && takes_few(P, xd, M);
+}
+static bool one_kernel(const gwq_packed* const* P, int count, gwq_dtype xd, int M) {
   for (int i = 1; i < count; ++i)
-    if (gwq_decode_ahead(P[i], xd, M) != rows) return GWQ_ERR_UNSUPPORTED;
-  return rows ? gwq_launch_decode_multi(P, count, x, xd, M, y, yd, stream) : gwq_launch_stream(P, count, x, xd, M, y, yd, stream);
+    if (gwq_decode_ahead(P[i], xd, M) != gwq_decode_ahead(P[0], xd, M)) return false;
+  return true;
+}
+// Layers that read the same x, up to 32 tokens, in one launch: the kernel that each layer takes by itself.  `scratch`: for
+// the copy of the activations that most kernels of several tokens make first, few_scratch bytes.
+static gwq_status launch_few(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M, void* const* y,
+                             gwq_dtype yd, void* scratch, cudaStream_t stream) {
+  if (!one_kernel(P, count, xd, M)) return GWQ_ERR_UNSUPPORTED;
+  return gwq_decode_ahead(P[0], xd, M) ? gwq_launch_decode_multi(P, count, x, xd, M, y, yd, scratch, stream)
+                                       : gwq_launch_stream(P, count, x, xd, M, y, yd, scratch, stream);
+}
+static size_t few_scratch(const gwq_packed* const* P, int count, gwq_dtype xd, int M) {
+  if (M > GWQ_DECODE_MAX_M || !one_kernel(P, count, xd, M)) return 0;
+  if (gwq_decode_ahead(P[0], xd, M) ? gwq_decode_stages(P, count, M) : M == 1 || !gwq_stream_takes(P[0], M)) return 0;
+  return gwq_stream_scratch_bytes(P[0]->K);
+}
+// the caller's workspace as that scratch
+static void* scratch_in(void* ws, size_t ws_bytes, size_t need) {
+  return need > 0 && ws && ws_bytes >= need && (reinterpret_cast<uintptr_t>(ws) & 255u) == 0 ? ws : nullptr;
+}
+static void* own_scratch(const gwq_packed* P) { return static_cast<const gwq_priv*>(P->priv)->xt; }
+
+// Calls without a workspace.  From nine tokens on they take the scratch inside the layer, so that calls on one layer have to
+// be ordered; with fewer they share nothing: where the kernel would need scratch, the tokens are taken a few at
+// a time, as many as the kernel with a CTA per tile stages in shared memory, or one by one.
+static const int kMostTokensAlone = 8;
+static gwq_status launch_alone(const gwq_packed* P, const void* x, gwq_dtype xd, int M, void* y, gwq_dtype yd, cudaStream_t stream) {
+  if (!takes_few(P, xd, M)) return GWQ_ERR_UNSUPPORTED;
+  if (few_scratch(&P, 1, xd, M) == 0) return launch_few(&P, 1, x, xd, M, &y, yd, nullptr, stream);
+  if (M > kMostTokensAlone) return launch_few(&P, 1, x, xd, M, &y, yd, own_scratch(P), stream);
+  for (int m = 0; m < M;) {
+    int n = M - m;
+    while (n > 1 && !gwq_decode_stages(&P, 1, n)) --n;
+    const char* const xm = static_cast<const char*>(x) + (size_t)m * P->K * dtype_bytes(xd);
+    void* const ym = static_cast<char*>(y) + (size_t)m * P->N * dtype_bytes(yd);
+    const gwq_status st = n > 1 ? gwq_launch_decode_multi(&P, 1, xm, xd, n, &ym, yd, nullptr, stream)
+                                : launch_few(&P, 1, xm, xd, 1, &ym, yd, nullptr, stream);
+    if (st != GWQ_OK) return st;
+    m += n;
+  }
+  return GWQ_OK;
 }
 
 extern "C" size_t gwq_linear_workspace_bytes(const gwq_packed* P, gwq_dtype xd, int32_t M) {
   if (!P || P->tag != GWQ_TAG_PACKED || !P->priv || M <= 0) return 0;
   if (wants_skinny(P, xd, M)) return gwq_skinny_workspace_bytes(P, M);
-  if (M <= GWQ_DECODE_MAX_M && takes_few(P, xd, M)) return 0;
+  if (M <= GWQ_DECODE_MAX_M && takes_few(P, xd, M)) return few_scratch(&P, 1, xd, M);
   return gwq_prefill_workspace_bytes(P, xd, M);
 }
 
@@ -45,7 +84,8 @@ extern "C" gwq_status gwq_linear_ws(const gwq_packed* P, const void* x, gwq_dtyp
   if (wants_skinny(P, xd, M) && ws && ws_bytes >= gwq_skinny_workspace_bytes(P, M))
     return gwq_launch_skinny(P, x, M, y, yd, ws, ws_bytes, stream);
   if (M <= GWQ_DECODE_MAX_M) {
-    const gwq_status st = launch_few(&P, 1, x, xd, M, &y, yd, stream);
+    void* const scratch = scratch_in(ws, ws_bytes, few_scratch(&P, 1, xd, M));
+    const gwq_status st = scratch ? launch_few(&P, 1, x, xd, M, &y, yd, scratch, stream) : launch_alone(P, x, xd, M, y, yd, stream);
     if (st != GWQ_ERR_UNSUPPORTED) return st;   // shapes they do not take: the tensor-core kernel
   }
   return gwq_launch_prefill(P, x, xd, M, y, yd, ws, ws_bytes, stream);
@@ -56,27 +96,58 @@ extern "C" gwq_status gwq_linear(const gwq_packed* P, const void* x, gwq_dtype x
   return gwq_linear_ws(P, x, xd, M, y, yd, nullptr, 0, stream_);
 }
 
-extern "C" gwq_status gwq_linear_multi(const gwq_packed* const* P, int32_t count, const void* x, gwq_dtype xd,
-                                       int32_t M, void* const* y, gwq_dtype yd, void* stream_) {
+// Several layers of up to 32 tokens as one launch: none of them takes the tcgen05 kernel by itself.
+static bool launches_as_one(const gwq_packed* const* P, int count, gwq_dtype xd, int M) {
+  for (int i = 0; i < count; ++i)
+    if (wants_skinny(P[i], xd, M)) return false;
+  return M <= GWQ_DECODE_MAX_M;
+}
+
+static bool valid_layers(const gwq_packed* const* P, int32_t count, int32_t M) {
+  if (!P || count < 1 || count > GWQ_MULTI_MAX || M <= 0) return false;
+  for (int i = 0; i < count; ++i)
+    if (!P[i] || P[i]->tag != GWQ_TAG_PACKED || !P[i]->S || !P[i]->priv || P[i]->K != P[0]->K) return false;
+  return true;
+}
+
+extern "C" size_t gwq_linear_multi_workspace_bytes(const gwq_packed* const* P, int32_t count, gwq_dtype xd, int32_t M) {
+  if (!valid_layers(P, count, M) || (xd != GWQ_F16 && xd != GWQ_BF16)) return 0;
+  size_t need = launches_as_one(P, count, xd, M) ? few_scratch(P, count, xd, M) : 0;
+  for (int i = 0; i < count; ++i) {
+    const size_t own = gwq_linear_workspace_bytes(P[i], xd, M);
+    need = own > need ? own : need;
+  }
+  return need;
+}
+
+extern "C" gwq_status gwq_linear_multi_ws(const gwq_packed* const* P, int32_t count, const void* x, gwq_dtype xd, int32_t M,
+                                          void* const* y, gwq_dtype yd, void* ws, size_t ws_bytes, void* stream_) {
   if (!P || !y || !x || count < 1 || count > GWQ_MULTI_MAX || M <= 0) return GWQ_ERR_INVALID_ARG;
   if (xd != GWQ_F16 && xd != GWQ_BF16) return GWQ_ERR_UNSUPPORTED;
   if (yd != GWQ_F16 && yd != GWQ_BF16 && yd != GWQ_F32) return GWQ_ERR_INVALID_ARG;
-  if (!gwq_aligned16(x)) return GWQ_ERR_INVALID_ARG;
-  for (int i = 0; i < count; ++i) {
-    if (!P[i] || P[i]->tag != GWQ_TAG_PACKED || !P[i]->S || !P[i]->priv || !y[i] || !gwq_aligned16(y[i]))
-      return GWQ_ERR_INVALID_ARG;
-    if (P[i]->K != P[0]->K) return GWQ_ERR_INVALID_ARG;
-  }
+  if (!gwq_aligned16(x) || !valid_layers(P, count, M)) return GWQ_ERR_INVALID_ARG;
+  for (int i = 0; i < count; ++i)
+    if (!y[i] || !gwq_aligned16(y[i])) return GWQ_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-  if (M <= GWQ_DECODE_MAX_M) {
-    const gwq_status st = launch_few(P, count, x, xd, M, y, yd, stream);
-    if (st != GWQ_ERR_UNSUPPORTED) return st;
+  if (M <= GWQ_DECODE_MAX_M && (!ws || launches_as_one(P, count, xd, M))) {
+    const size_t need = few_scratch(P, count, xd, M);
+    void* scratch = scratch_in(ws, ws_bytes, need);
+    if (!scratch && M > kMostTokensAlone) scratch = own_scratch(P[0]);
+    if (scratch || need == 0) {
+      const gwq_status st = launch_few(P, count, x, xd, M, y, yd, scratch, stream);
+      if (st != GWQ_ERR_UNSUPPORTED) return st;
+    }
   }
   for (int i = 0; i < count; ++i) {   // more tokens than the streaming kernel takes, or layers of different kinds
-    const gwq_status st = gwq_linear(P[i], x, xd, M, y[i], yd, stream_);
+    const gwq_status st = gwq_linear_ws(P[i], x, xd, M, y[i], yd, ws, ws_bytes, stream_);
     if (st != GWQ_OK) return st;
   }
   return GWQ_OK;
+}
+
+extern "C" gwq_status gwq_linear_multi(const gwq_packed* const* P, int32_t count, const void* x, gwq_dtype xd,
+                                       int32_t M, void* const* y, gwq_dtype yd, void* stream_) {
+  return gwq_linear_multi_ws(P, count, x, xd, M, y, yd, nullptr, 0, stream_);
 }
 
 // A staging buffer of at least `need` bytes; its last use was on whatever stream the caller had then.
@@ -120,13 +191,13 @@ static gwq_status linear_host(gwq_packed* P, const void* x_host, gwq_dtype xd, i
   // transposing pre-pass, or, where every CTA reads them, by a kernel that copies them first) and y is
   // written once, so that nothing is gained by the copy engine, whose two copies take longer than the product
   // (4096 x 11008 at 4 tokens: 47 -> 34 us).
-  const bool direct = M <= GWQ_DECODE_MAX_M && !wants_skinny(P, xd, M) && takes_few(P, xd, M);
+  const bool direct = gwq_takes_decode(P, xd, M);
   const bool copied = M == 1 || (direct && gwq_decode_ahead(P, xd, M));
   const void* x = direct && gwq_aligned16(x_host) ? device_view(x_host, xb) : nullptr;
   void* y = direct && yb <= kDirectMostBytes ? device_view(y_host, yb) : nullptr;
   if (!x || copied) GWQ_CUDA_TRY(grow(&pv->x_stage, &pv->x_stage_bytes, xb, stream));
   if (!y) GWQ_CUDA_TRY(grow(&pv->y_stage, &pv->y_stage_bytes, yb, stream));
-  GWQ_CUDA_TRY(grow(&pv->ws_stage, &pv->ws_stage_bytes, gwq_linear_workspace_bytes(P, xd, M), stream));
+  if (!direct) GWQ_CUDA_TRY(grow(&pv->ws_stage, &pv->ws_stage_bytes, gwq_linear_workspace_bytes(P, xd, M), stream));
   if (!x) {
     GWQ_CUDA_TRY(cudaMemcpyAsync(pv->x_stage, x_host, xb, cudaMemcpyHostToDevice, stream));
   } else if (copied) {
@@ -135,7 +206,7 @@ static gwq_status linear_host(gwq_packed* P, const void* x_host, gwq_dtype xd, i
   if (!x || copied) x = pv->x_stage;
   if (direct) {
     void* const out = y ? y : pv->y_stage;
-    st = launch_few(&P, 1, x, xd, M, &out, yd, stream);
+    st = launch_few(&P, 1, x, xd, M, &out, yd, own_scratch(P), stream);
   } else {
     st = gwq_linear_ws(P, x, xd, M, pv->y_stage, yd, pv->ws_stage, pv->ws_stage_bytes, stream);
   }

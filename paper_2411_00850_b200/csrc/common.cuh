@@ -34,7 +34,7 @@ struct gwq_priv {
                          // [group of the step][row >> 3], rows past the last one zero (NULL where it takes no call)
   void* ws_stage;        // scratch for gwq_linear_host where the product needs some
   size_t ws_stage_bytes;
-  void* xt;              // scratch of the decode kernels: transposed activations
+  void* xt;              // scratch of the decode kernels (transposed activations) for calls without a workspace
   uint32_t* ob;          // outliers ordered by block of 128 rows x 128 columns: row << 23 | column << 16 | fp16 value
   uint32_t* tb;          // outliers ordered by tile of 16 rows and step of 128 columns: fp16 value << 16 | column << 4 | row
   int32_t* tb_ptr;       // [tiles * steps + 1] extents of the blocks in tb (K a multiple of 128)
@@ -83,8 +83,10 @@ void gwq_delete_outliers(gwq_outliers* S);
 // Kernel launchers implemented in the other translation units.
 gwq_status gwq_launch_simt(const gwq_packed* P, const void* x, gwq_dtype xd, int M, void* y,
                            gwq_dtype yd, cudaStream_t stream);
+// scratch: gwq_stream_scratch_bytes, not read where every layer's activations are staged (and with one token)
 gwq_status gwq_launch_decode_multi(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M,
-                                   void* const* y, gwq_dtype yd, cudaStream_t stream);
+                                   void* const* y, gwq_dtype yd, void* scratch, cudaStream_t stream);
+bool gwq_decode_stages(const gwq_packed* const* P, int count, int M);   // it serves the call without scratch
 bool gwq_decode_ahead(const gwq_packed* P, gwq_dtype xd, int M);   // the kernel with a CTA per tile is the faster one for (P, xd, M)
 gwq_status gwq_launch_prefill(const gwq_packed* P, const void* x, gwq_dtype xd, int M, void* y,
                               gwq_dtype yd, void* ws, size_t ws_bytes, cudaStream_t stream);
@@ -93,7 +95,8 @@ bool gwq_skinny_takes(const gwq_packed* P, gwq_dtype xd, int M);
 size_t gwq_skinny_workspace_bytes(const gwq_packed* P, int M);
 gwq_status gwq_launch_skinny(const gwq_packed* P, const void* x, int M, void* y, gwq_dtype yd, void* ws, size_t ws_bytes,
                              cudaStream_t stream);
+bool gwq_takes_decode(const gwq_packed* P, gwq_dtype xd, int M);   // one of the two decode kernels serves (P, xd, M)
 bool gwq_stream_takes(const gwq_packed* P, int M);   // the streaming kernel has a variant for (P, M)
-size_t gwq_stream_scratch_bytes(int K);              // bytes of gwq_priv::xt it needs
+size_t gwq_stream_scratch_bytes(int K);              // scratch of a call of several tokens, for either decode kernel
 gwq_status gwq_launch_stream(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M, void* const* y,
-                             gwq_dtype yd, cudaStream_t stream);
+                             gwq_dtype yd, void* scratch, cudaStream_t stream);

@@ -193,10 +193,16 @@ bool gwq_decode_ahead(const gwq_packed* P, gwq_dtype xd, int M) {
   return g128 && lone;   // 0.92 to 0.97
 }
 
+bool gwq_decode_stages(const gwq_packed* const* P, int count, int M) {
+  Variant v;
+  int cvcap;
+  return plan(P, count, M, &v, &cvcap) && (v.nbuf == 0 || v.tp == 1);
+}
+
 // Decode launcher for `count` layers that read the same x.  Returns GWQ_ERR_UNSUPPORTED where the streaming kernel
-// has no variant (nothing has been launched then).  The scratch for the token-major copy of x is the first layer's.
+// has no variant (nothing has been launched then).  A token-major copy of x goes to `scratch`.
 gwq_status gwq_launch_decode_multi(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M,
-                                   void* const* y, gwq_dtype yd, cudaStream_t stream) {
+                                   void* const* y, gwq_dtype yd, void* scratch, cudaStream_t stream) {
   Variant v;
   MultiArgs a;
   if (!plan(P, count, M, &v, &a.cvcap)) return GWQ_ERR_UNSUPPORTED;
@@ -219,8 +225,9 @@ gwq_status gwq_launch_decode_multi(const gwq_packed* const* P, int count, const 
   a.sm_count = pv->sm_count > 0 ? pv->sm_count : 148;
   a.x = static_cast<const uint16_t*>(x); a.yd = yd; a.K = K; a.M = M;
   if (v.nbuf != 0 && v.tp > 1) {   // token-major copy of x and its group sums, once for all layers
-    uint16_t* xt = static_cast<uint16_t*>(pv->xt);
-    float* xg = reinterpret_cast<float*>(static_cast<char*>(pv->xt) + (size_t)K * 32 * 2);
+    if (!scratch) return GWQ_ERR_WORKSPACE;
+    uint16_t* xt = static_cast<uint16_t*>(scratch);
+    float* xg = reinterpret_cast<float*>(static_cast<char*>(scratch) + (size_t)K * 32 * 2);
     const bool bf = xd == GWQ_BF16;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

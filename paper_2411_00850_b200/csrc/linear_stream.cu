@@ -147,9 +147,9 @@ bool gwq_stream_takes(const gwq_packed* P, int M) {
 }
 
 // `count` layers that read the same x, in one launch.  GWQ_ERR_UNSUPPORTED where the kernel has no variant (nothing has
-// been launched then).  The transposed activations go to the first layer's scratch.
+// been launched then).  The transposed activations of several tokens go to `scratch`.
 gwq_status gwq_launch_stream(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M, void* const* y,
-                             gwq_dtype yd, cudaStream_t stream) {
+                             gwq_dtype yd, void* scratch, cudaStream_t stream) {
   Variant v;
   int first_cta[kMaxLayers], grid;
   if (!plan(P, count, M, &v, first_cta, &grid)) return GWQ_ERR_UNSUPPORTED;
@@ -168,7 +168,8 @@ gwq_status gwq_launch_stream(const gwq_packed* const* P, int count, const void* 
   const bool bf = xd == GWQ_BF16;
   cudaError_t e = cudaSuccess;
   if (v.tp > 1) {
-    unsigned char* xt = static_cast<unsigned char*>(static_cast<const gwq_priv*>(P[0]->priv)->xt);
+    unsigned char* xt = static_cast<unsigned char*>(scratch);
+    if (!xt) return GWQ_ERR_WORKSPACE;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

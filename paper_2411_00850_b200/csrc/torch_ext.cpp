@@ -16,6 +16,7 @@
 
 #include "../../include/gwq.h"
 
+bool gwq_takes_decode(const gwq_packed* P, gwq_dtype xd, int M);
 cudaError_t gwq_copy_arrays(int count, const void* const* from, void* const* to, const size_t* bytes, cudaStream_t stream);
 
 namespace {
@@ -196,23 +197,29 @@ PyObject* py_linear_multi(PyObject*, PyObject* const* a, Py_ssize_t n) {
     for (const at::Tensor& o : outs) fits = fits && o.scalar_type() == outs[0].scalar_type();
     if (!fits) fail(PyExc_ValueError, "one output per layer, all of one dtype");
     const gwq_dtype xd = dtype_code(x.scalar_type());
-    size_t need = 0;
-    for (Py_ssize_t i = 0; i < count && xd != GWQ_F32; ++i)
-      need = std::max(need, gwq_linear_workspace_bytes(P[i], xd, (int32_t)x.size(0)));
+    const int32_t M = (int32_t)x.size(0);
     const cudaStream_t stream = at::cuda::getCurrentCUDAStream();
-    if (need > 0) {   // products that take scratch memory: one call per layer, all on one workspace (stream order)
-      const at::Tensor ws = workspace_for(a[4], need, x.device());
+    // more layers than one call takes: one by one, on one workspace (stream order), where it is the tensor-core kernels that want it
+    size_t alone = 0;
+    for (Py_ssize_t i = 0; i < count && count > GWQ_MULTI_MAX && xd != GWQ_F32; ++i)
+      if (!gwq_takes_decode(P[i], xd, M)) alone = std::max(alone, gwq_linear_workspace_bytes(P[i], xd, M));
+    if (alone > 0) {
+      for (Py_ssize_t i = 0; i < count; ++i) alone = std::max(alone, gwq_linear_workspace_bytes(P[i], xd, M));
+      const at::Tensor ws = workspace_for(a[4], alone, x.device());
       for (Py_ssize_t i = 0; i < count; ++i) run_linear(P[i], x, xd, outs[i], ws, stream);
     } else {
       std::vector<void*> y(std::max<Py_ssize_t>(count, 1), nullptr);
       for (Py_ssize_t i = 0; i < count; ++i) y[i] = outs[i].data_ptr();
       const gwq_dtype yd = count ? dtype_code(outs[0].scalar_type()) : GWQ_F16;
       const void* px = x.data_ptr();
-      gwq_status st;
       P.resize(std::max<Py_ssize_t>(count, 1), nullptr);
+      const at::Tensor ws = workspace_for(a[4], gwq_linear_multi_workspace_bytes(P.data(), (int32_t)count, xd, M), x.device());
+      void* pw = ws.defined() ? ws.data_ptr() : nullptr;
+      const size_t wb = ws.defined() ? bytes_of(ws) : 0;
+      gwq_status st;
       {
         no_gil released;
-        st = gwq_linear_multi(P.data(), (int32_t)count, px, xd, (int32_t)x.size(0), y.data(), yd, stream);
+        st = gwq_linear_multi_ws(P.data(), (int32_t)count, px, xd, M, y.data(), yd, pw, wb, stream);
       }
       check(st, "gwq_linear_multi");
     }
