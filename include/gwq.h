@@ -209,7 +209,7 @@ gwq_status gwq_gradient_mean(const float* const* G_list, int32_t count, int64_t 
  * ||W - W_Q||_2^2 (Eq. "Q") and the first-order change of the loss g^T (W - W_Q) (Eq. "Taylor",
  * Eq. "final_OPO"), with W_Q = s (q - z) + S as gwq_linear uses it.  Terms and sums in FP64, in a fixed
  * order.  W_f16 [N,K], G_f32 [N,K]: device, the arrays P was made from (any other pair of that shape gives
- * the same formulas on them).  *sq_err, *first_order: host.  Allocates 16 N bytes for the call,
+ * the same formulas on them); any element-aligned address, 16-byte aligned ones are read faster.  *sq_err, *first_order: host.  Allocates 16 N bytes for the call,
  * synchronises `stream`.  Errors: INVALID_ARG, ALLOC, CUDA.                                             */
 gwq_status gwq_quality(const uint16_t* W_f16, const float* G_f32, const gwq_packed* P, double* sq_err,
                        double* first_order, void* stream);

@@ -56,8 +56,8 @@ struct Eight {
 // and handled from the CSR entries instead.  s (q - z) has at most 20 bits: the FP32 product is exact.
 // Bound by memory latency and the FP64 conversions (a third of the conversion unit).  11008 x 4096: one thread per run
 // of 32 columns with 2- and 4-byte loads 291 us, one CTA per row with these loads 103 (waiting at its
-// barriers), this 73.
-template <int BITS>
+// barriers), this 73.  WIDE: W and G start on 16 bytes (a view of a larger buffer need not: element loads then).
+template <int BITS, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 5)
 quality_row_kernel(const uint16_t* __restrict__ W, const float* __restrict__ G, const uint32_t* __restrict__ codes,
                    const uint16_t* __restrict__ scales, const uint8_t* __restrict__ zeros,
@@ -73,8 +73,6 @@ quality_row_kernel(const uint16_t* __restrict__ W, const float* __restrict__ G, 
   const uint32_t* crow = codes + (size_t)n * nruns * BITS;
   const uint16_t* srow = scales + (size_t)n * ngroups;
   const uint8_t* zrow = zeros + (size_t)n * ngroups;
-  const uint4* w4 = reinterpret_cast<const uint4*>(wrow);
-  const float4* g4 = reinterpret_cast<const float4*>(grow);
   uint4 w[kAhead];
   float4 ga[kAhead], gb[kAhead];
   Eight<BITS> packed[kAhead];
@@ -82,9 +80,17 @@ quality_row_kernel(const uint16_t* __restrict__ W, const float* __restrict__ G, 
   const int shift = 31 - __clz(group);
   auto fetch = [&](const int u, const int i) {
     if (i < n8) {
-      w[u] = __ldcs(w4 + i);
-      ga[u] = __ldcs(g4 + 2 * i);
-      gb[u] = __ldcs(g4 + 2 * i + 1);
+      if constexpr (WIDE) {
+        w[u] = __ldcs(reinterpret_cast<const uint4*>(wrow) + i);
+        ga[u] = __ldcs(reinterpret_cast<const float4*>(grow) + 2 * i);
+        gb[u] = __ldcs(reinterpret_cast<const float4*>(grow) + 2 * i + 1);
+      } else {
+        auto pair = [&](const int e) { return (unsigned)wrow[8 * i + e] | (unsigned)wrow[8 * i + e + 1] << 16; };
+        const float* g = grow + 8 * i;
+        w[u] = make_uint4(pair(0), pair(2), pair(4), pair(6));
+        ga[u] = make_float4(g[0], g[1], g[2], g[3]);
+        gb[u] = make_float4(g[4], g[5], g[6], g[7]);
+      }
       packed[u].fetch(crow + (i >> 2) * BITS, i & 3);
       scale[u] = __ldg(srow + ((i * 8) >> shift)) | (unsigned)__ldg(zrow + ((i * 8) >> shift)) << 16;
     }
@@ -165,6 +171,7 @@ __global__ void __launch_bounds__(1024) quality_sum_kernel(const double* __restr
 extern "C" gwq_status gwq_quality(const uint16_t* W, const float* G, const gwq_packed* P, double* sq_err,
                                   double* first_order, void* stream_) {
   if (!W || !G || !P || P->tag != GWQ_TAG_PACKED || !P->S || !sq_err || !first_order) return GWQ_ERR_INVALID_ARG;
+  if ((reinterpret_cast<uintptr_t>(W) & 1u) != 0 || (reinterpret_cast<uintptr_t>(G) & 3u) != 0) return GWQ_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   gwq_status st = GWQ_OK;
   void* scratch = nullptr;
@@ -174,17 +181,24 @@ extern "C" gwq_status gwq_quality(const uint16_t* W, const float* G, const gwq_p
   if (!host) return GWQ_ERR_ALLOC;
   GWQ_CUDA_TRY(gwq_dev_alloc(&scratch, (size_t)P->N * 2 * sizeof(double), stream));
   rows = static_cast<double*>(scratch);
-#define GWQ_QUALITY_LAUNCH(BITS)                                                                                     \
+#define GWQ_QUALITY_LAUNCH(BITS, WIDE)                                                                               \
   do {                                                                                                               \
-    GWQ_CUDA_TRY(cudaFuncSetAttribute(quality_row_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
+    GWQ_CUDA_TRY(cudaFuncSetAttribute(quality_row_kernel<BITS, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                       (int)smem));                                                                   \
-    quality_row_kernel<BITS><<<(P->N + kThreads / 32 - 1) / (kThreads / 32), kThreads, smem, stream>>>(              \
+    quality_row_kernel<BITS, WIDE><<<(P->N + kThreads / 32 - 1) / (kThreads / 32), kThreads, smem, stream>>>(        \
         W, G, P->codes, P->scales, P->zeros, P->S->row_ptr, P->S->col_idx, P->S->val, P->N, P->K, P->group, rows);   \
   } while (0)
-  if (P->bits == 4) GWQ_QUALITY_LAUNCH(4);
-  else if (P->bits == 3) GWQ_QUALITY_LAUNCH(3);
-  else if (P->bits == 8) GWQ_QUALITY_LAUNCH(8);
-  else GWQ_QUALITY_LAUNCH(2);
+  if (gwq_aligned16(W) && gwq_aligned16(G)) {
+    if (P->bits == 4) GWQ_QUALITY_LAUNCH(4, true);
+    else if (P->bits == 3) GWQ_QUALITY_LAUNCH(3, true);
+    else if (P->bits == 8) GWQ_QUALITY_LAUNCH(8, true);
+    else GWQ_QUALITY_LAUNCH(2, true);
+  } else {
+    if (P->bits == 4) GWQ_QUALITY_LAUNCH(4, false);
+    else if (P->bits == 3) GWQ_QUALITY_LAUNCH(3, false);
+    else if (P->bits == 8) GWQ_QUALITY_LAUNCH(8, false);
+    else GWQ_QUALITY_LAUNCH(2, false);
+  }
 #undef GWQ_QUALITY_LAUNCH
   GWQ_CUDA_TRY(cudaGetLastError());
   quality_sum_kernel<<<1, 1024, 0, stream>>>(rows, P->N, host);
