@@ -214,15 +214,16 @@ gwq_status gwq_gradient_mean(const float* const* G_list, int32_t count, int64_t 
 gwq_status gwq_quality(const uint16_t* W_f16, const float* G_f32, const gwq_packed* P, double* sq_err,
                        double* first_order, void* stream);
 
-/* Same product with HOST buffers: copies x_host [M,K] to a staging buffer kept inside P,
- * runs gwq_linear, copies y back into y_host [M,N] and synchronises `stream`.
+/* Same product with HOST buffers, x_host [M,K] and y_host [M,N], at any address; synchronises `stream` before it returns.
+ * x_host is copied to a staging buffer kept inside P, and y back from one; up to 32 tokens the decode kernels read and
+ * write page-locked buffers themselves instead (x_host 16-byte aligned, y_host aligned to its elements and up to 256 KB).
  * For best copy speed the host buffers should be page-locked.  The staging buffers (and the scratch
- * of gwq_linear_ws, where needed) grow on demand (cudaMalloc) and are shared by all calls on P: not
+ * of gwq_linear_ws, where needed) grow on demand (from the library's memory pool) and are shared by all calls on P: not
  * re-entrant per P.                                                                    */
 gwq_status gwq_linear_host(gwq_packed* P, const void* x_host, gwq_dtype x_dtype, int32_t M,
                            void* y_host, gwq_dtype y_dtype, void* stream);
 
-/* gwq_linear_host without the final synchronisation: the copy of x, the product and the copy of y are
+/* gwq_linear_host without the final synchronisation: the copies, if any, and the product are
  * enqueued on `stream` and the call returns; y_host is valid, and x_host may be reused, once the caller
  * has synchronised the stream (one synchronisation can serve many calls).  Calls that share P must be
  * on one stream (they share P's staging buffers, and stream order keeps them apart).  Use page-locked

@@ -194,7 +194,9 @@ static gwq_status linear_host(gwq_packed* P, const void* x_host, gwq_dtype xd, i
   const bool direct = gwq_takes_decode(P, xd, M);
   const bool copied = M == 1 || (direct && gwq_decode_ahead(P, xd, M));
   const void* x = direct && gwq_aligned16(x_host) ? device_view(x_host, xb) : nullptr;
-  void* y = direct && yb <= kDirectMostBytes ? device_view(y_host, yb) : nullptr;
+  // (the kernels store element by element; the copy engine takes any address)
+  const bool whole = (reinterpret_cast<uintptr_t>(y_host) & (dtype_bytes(yd) - 1)) == 0;
+  void* y = direct && whole && yb <= kDirectMostBytes ? device_view(y_host, yb) : nullptr;
   if (!x || copied) GWQ_CUDA_TRY(grow(&pv->x_stage, &pv->x_stage_bytes, xb, stream));
   if (!y) GWQ_CUDA_TRY(grow(&pv->y_stage, &pv->y_stage_bytes, yb, stream));
   if (!direct) GWQ_CUDA_TRY(grow(&pv->ws_stage, &pv->ws_stage_bytes, gwq_linear_workspace_bytes(P, xd, M), stream));
