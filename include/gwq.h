@@ -27,6 +27,7 @@
 #ifndef GWQ_H_
 #define GWQ_H_
 
+#include <stddef.h>
 #include <stdint.h>
 
 #ifdef __cplusplus
@@ -248,6 +249,12 @@ gwq_status gwq_set_wait_limit(gwq_packed* P, int64_t cycles);
 
 /* Releases a gwq_outliers* or a gwq_packed* (and everything it owns).  NULL is a no-op. */
 void gwq_free(void* obj);
+
+/* Gives memory that the library keeps for its next objects on the current device back to the system, down to keep_bytes.
+ * Objects live in one memory pool per device, which keeps up to 256 MB of what gwq_free released (an allocation from it
+ * takes about a microsecond); the process's other allocators cannot reach that memory.  Memory in use is untouched.
+ * Synchronises the device; not during stream capture.  Errors: CUDA.                                   */
+gwq_status gwq_trim_memory(size_t keep_bytes);
 
 /* Static, NUL-terminated name of a status code.                                        */
 const char* gwq_status_string(gwq_status s);

@@ -29,7 +29,8 @@ STATUS_NAMES = {
 }
 EXPORTS = ("gwq_select_outliers", "gwq_select_outliers_static", "gwq_outliers_rows", "gwq_pack", "gwq_linear", "gwq_linear_ws",
            "gwq_linear_workspace_bytes", "gwq_linear_multi", "gwq_linear_multi_ws", "gwq_linear_multi_workspace_bytes",
-           "gwq_gradient_mean", "gwq_quality", "gwq_linear_host", "gwq_linear_host_async", "gwq_device_status", "gwq_set_wait_limit", "gwq_free", "gwq_status_string")
+           "gwq_gradient_mean", "gwq_quality", "gwq_linear_host", "gwq_linear_host_async", "gwq_device_status", "gwq_set_wait_limit", "gwq_free",
+           "gwq_trim_memory", "gwq_status_string")
 GWQ_MULTI_MAX = 4
 
 
@@ -106,6 +107,8 @@ def load_library(path: str = LIB_PATH) -> C.CDLL:
     lib.gwq_set_wait_limit.argtypes = [C.POINTER(gwq_packed), C.c_int64]
     lib.gwq_free.restype = None
     lib.gwq_free.argtypes = [C.c_void_p]
+    lib.gwq_trim_memory.restype = C.c_int
+    lib.gwq_trim_memory.argtypes = [C.c_size_t]
     lib.gwq_status_string.restype = C.c_char_p
     lib.gwq_status_string.argtypes = [C.c_int]
     _lib = lib
@@ -318,3 +321,9 @@ def gwq_set_wait_limit(P: Packed, cycles: int) -> None:
 
 def gwq_free(obj) -> None:
     obj.free()
+
+
+def gwq_trim_memory(keep_bytes: int = 0, device=None) -> None:
+    """Give memory that the library keeps for its next objects (at most 256 MB a device) back to the system."""
+    with torch.cuda.device(device):
+        _check(int(load_library().gwq_trim_memory(int(keep_bytes))), "gwq_trim_memory")

@@ -3,7 +3,8 @@
 // Objects live in one stream-ordered pool per device: a cudaMalloc / cudaFree pair of a layer's arrays takes hundreds
 // of microseconds (encoding a 4096 x 4096 layer spent 1.9 of 2.2 ms in them), an allocation that the pool can serve
 // about one.  The pool keeps at most kPoolKeepBytes of unused memory; what is above goes back to the system at the
-// next synchronisation, and all of it when an allocation fails.
+// next synchronisation, all of it when an allocation fails, and whatever the caller asks for through gwq_trim_memory
+// (other allocators of the process cannot reach it).
 #include <mutex>
 #include <vector>
 
@@ -62,6 +63,26 @@ cudaError_t gwq_dev_alloc(void** p, size_t bytes, cudaStream_t stream) {
     e = cudaMallocFromPoolAsync(p, bytes, pool, stream);
   }
   return e;
+}
+
+extern "C" gwq_status gwq_trim_memory(size_t keep_bytes) {
+  int dev = -1;
+  cudaMemPool_t pool = nullptr;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return GWQ_ERR_CUDA;
+  }
+  if (dev >= 0 && dev < kMaxDevices) {
+    std::lock_guard<std::mutex> lock(g_mutex);
+    pool = g_pool[dev];
+  }
+  if (!pool) return GWQ_OK;   // nothing has been allocated on this device
+  // what was freed in stream order is unused once the frees have been reached
+  if (cudaDeviceSynchronize() != cudaSuccess || cudaMemPoolTrimTo(pool, keep_bytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return GWQ_ERR_CUDA;
+  }
+  return GWQ_OK;
 }
 
 void gwq_dev_free_async(void* p, cudaStream_t stream) {
