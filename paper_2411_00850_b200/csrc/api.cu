@@ -8,13 +8,9 @@
 
 static size_t dtype_bytes(gwq_dtype d) { return d == GWQ_F32 ? 4 : 2; }
 
-// 17 to 32 fp16 tokens with a workspace: the tcgen05 streaming kernel for small layers and, with 3 bits, for large ones
-// (24 tokens, its time to the mma.sync streaming kernel's: 0.83 on 10240 x 10240, 0.79 on 3000 x 24064, 0.94 on 28672 x
-// 8192; 1.0 to 1.3 on layers in between, 1.1 to 1.5 with 4 bits).
+// 17 to 32 fp16 tokens with a workspace: the tcgen05 streaming kernel, for the layers that gwq_pack made its list for.
 static bool wants_skinny(const gwq_packed* P, gwq_dtype xd, int M) {
-  const long long weights = (long long)P->N * P->K;
-  return (weights <= GWQ_SKINNY_MOST_WEIGHTS || (P->bits == 3 && weights > 72LL * 1000 * 1000)) && M >= 17 && M <= GWQ_DECODE_MAX_M &&
-         gwq_skinny_takes(P, xd, M);
+  return M >= 17 && M <= GWQ_DECODE_MAX_M && gwq_skinny_takes(P, xd, M);
 }
 
 static bool takes_few(const gwq_packed* P, gwq_dtype xd, int M) { return gwq_decode_ahead(P, xd, M) || gwq_stream_takes(P, M); }

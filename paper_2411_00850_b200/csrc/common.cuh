@@ -44,8 +44,6 @@ struct gwq_priv {
   long long wait_cycles; // SM cycles a bounded device-side wait may spin (gwq_set_wait_limit)
 };
 
-// layers of up to this many weights take the tcgen05 streaming kernel for 17 to 32 fp16 tokens
-#define GWQ_SKINNY_MOST_WEIGHTS (5LL * 1024 * 1024)
 #define GWQ_DEFAULT_WAIT_CYCLES (1000LL * 1000LL * 1000LL)
 
 static inline bool gwq_aligned16(const void* p) {
@@ -91,6 +89,7 @@ bool gwq_decode_ahead(const gwq_packed* P, gwq_dtype xd, int M);   // the kernel
 gwq_status gwq_launch_prefill(const gwq_packed* P, const void* x, gwq_dtype xd, int M, void* y,
                               gwq_dtype yd, void* ws, size_t ws_bytes, cudaStream_t stream);
 size_t gwq_prefill_workspace_bytes(const gwq_packed* P, gwq_dtype xd, int M);
+bool gwq_skinny_layer(const gwq_packed* P);   // takes the tcgen05 streaming kernel for 17 to 32 fp16 tokens: gwq_pack makes its list
 bool gwq_skinny_takes(const gwq_packed* P, gwq_dtype xd, int M);
 size_t gwq_skinny_workspace_bytes(const gwq_packed* P, int M);
 gwq_status gwq_launch_skinny(const gwq_packed* P, const void* x, int M, void* y, gwq_dtype yd, void* ws, size_t ws_bytes,

@@ -646,11 +646,38 @@ gwq_status launch(const gwq_packed* P, const void* x, int M, void* y, gwq_dtype 
 
 }  // namespace
 
-// The skinny kernel takes fp16 activations, up to 32 tokens, groups of 64 or 128, K a multiple of 128 up to 65536.
+// Which layers take this kernel (17 to 32 fp16 tokens); gwq_pack asks too, and makes the outliers' list by blocks for these.
+//  * 3 bits in groups of 64: the mma.sync streaming kernel keeps such groups apart by columns and has none left beyond 16
+//    tokens, and the kernel after that rounds the scaled weights to fp16 (24 tokens, error of y 1.6e-4 against 3e-6; us:
+//    42.9 -> 19.5 on 4096 x 4096, 220 -> 60 on 3000 x 24064, 80 -> 55 on 8192 x 8192, 153 -> 187 on 28672 x 8192).
+//  * Groups of 128: where its even shares of the layer (stream-K over blocks of 128 x 128) make up for its pipeline's
+//    start-up and its second kernel.  Microseconds, with G steps of 128 columns, a tiles of 16 rows per SM and n = ceil(a)
+//    of them for the busiest SM, 24 tokens:
+//      here 9.5 + 0.1325 a G;  the streaming kernel 4.5 + c n G, with c the cost of a tile and step: c = 0.115 up
+//      to four tiles (one pass), 0.145 at five (two passes), 0.12 beyond (sixteen warps) with 4 bits; 0.13 up to four,
+//      0.147 beyond with 3 bits.
+//    Within 10 % of both kernels' times on 13 layers of 16 M weights and more, and on the faster one's side but where the two
+//    differ by 2 %: 4 bits 3000 x 24064 51.2 -> 43.6, 10240 x 10240 61.0 -> 54.2 (not: 8192 x 8192 32.5 / 37.6, 28672 x 8192
+//    96.5 / 113); 3 bits 3000 x 24064 55.1 -> 43.1, 10240 x 10240 67.5 -> 53.7, 28672 x 8192 121.6 -> 112.5, 8192 x 28672
+//    119.3 -> 107.8, 20480 x 5120 59.0 -> 57.0 (not: 8192 x 8192 36.1 / 37.0, 13824 x 5120 40.0 / 41.9).  Groups of 64 with 4
+//    bits take two accumulators per step here and are slower (38 / 54 on 8192 x 8192).
+//  * Layers of up to 5 M weights, although the streaming kernel has come to be ahead there too (4.7 / 9.7 on 1024 x 1024,
+//    9.2 / 13.5 on 1024 x 4096).
+bool gwq_skinny_layer(const gwq_packed* P) {
+  const gwq_priv* pv = static_cast<const gwq_priv*>(P->priv);
+  if ((P->bits != 3 && P->bits != 4) || (P->group != 64 && P->group != 128) || P->K % 128 != 0 || P->K > 65536) return false;
+  if (P->bits == 3 && P->group == 64) return true;
+  if ((long long)P->N * P->K <= 5LL * 1024 * 1024) return true;
+  if (P->group == 64) return false;
+  const int sms = pv->sm_count > 0 ? pv->sm_count : 148, tiles = (P->N + 15) / 16, n = (tiles + sms - 1) / sms, G = P->K / 128;
+  const double c = P->bits == 3 ? (n <= 4 ? 0.13 : 0.147) : (n <= 4 ? 0.115 : tiles <= 5 * sms ? 0.145 : 0.12);
+  return 9.5 + 0.1325 * tiles / sms * G < 4.5 + c * n * G;
+}
+
+// The skinny kernel takes fp16 activations, up to 32 tokens.
 bool gwq_skinny_takes(const gwq_packed* P, gwq_dtype xd, int M) {
   const gwq_priv* pv = static_cast<const gwq_priv*>(P->priv);
-  return xd == GWQ_F16 && (P->bits == 3 || P->bits == 4) && M >= 1 && M <= 32 && (P->group == 64 || P->group == 128) && P->K % 128 == 0 && P->K <= 65536 &&
-         pv->ob && pv->ob_ptr && pv->sz_t;
+  return xd == GWQ_F16 && M >= 1 && M <= 32 && pv->ob && pv->ob_ptr && pv->sz_t && gwq_skinny_layer(P);
 }
 
 // Workspace: two partial tiles per CTA.

@@ -158,7 +158,7 @@ constexpr int kSlice = 32;   // groups of one transposing CTA
 //   cv  one word per outlier in CSR order: fp16 value << 16 | column;
 //   tb  the same outliers ordered by tile of 16 rows and step of 128 columns (tile * (K / 128) + step), inside by row and
 //       column: value << 16 | column of the step << 4 | row of the tile; tb_ptr[b] .. tb_ptr[b + 1] are the entries of b;
-//   ob  (small layers only) ordered by block of 128 rows x 128 columns: row-in-block << 23 | column-in-block << 16 |
+//   ob  (layers of the tcgen05 streaming kernel) ordered by block of 128 rows x 128 columns: row-in-block << 23 | column-in-block << 16 |
 //       value, with ob_ptr likewise (the order inside a block is whatever the atomics give; its reader places every entry
 //       by its position).
 //   The entries of 128 rows are one stretch of the CSR arrays and of both lists, so counting, scanning and filling stay
@@ -311,9 +311,9 @@ cudaError_t launch_pack(int group, const uint16_t* W, const gwq_outliers* S, int
 // The layer's arrays, all in one allocation that starts with the codes.
 void carve(gwq_carver& c, gwq_packed* P, gwq_priv* pv, int64_t nnz) {
   const size_t ngroups = (size_t)P->N * (P->K / P->group);
-  const bool lists = P->K <= 65536, blocks = lists && P->group >= 64 && P->K % 128 == 0;
+  const bool lists = P->K <= 65536, blocks = gwq_skinny_layer(P);
   // whole tiles of 16 rows: the streaming kernel reads (and gives weight zero to) the rows past the last one
-  const bool tiles = lists && P->K % 128 == 0, small = blocks && (long long)P->N * P->K <= GWQ_SKINNY_MOST_WEIGHTS;
+  const bool tiles = lists && P->K % 128 == 0;
   P->codes = c.take<uint32_t>((size_t)(P->N + 15) / 16 * 16 * (P->K / 32) * P->bits);
   P->scales = c.take<uint16_t>(ngroups + 8);
   P->zeros = c.take<uint8_t>(ngroups + 16);
@@ -323,8 +323,8 @@ void carve(gwq_carver& c, gwq_packed* P, gwq_priv* pv, int64_t nnz) {
   pv->cv = lists ? c.take<uint32_t>((size_t)nnz + 4) : nullptr;
   pv->tb = tiles ? c.take<uint32_t>((size_t)nnz + 4) : nullptr;
   pv->tb_ptr = tiles ? c.take<int32_t>((size_t)((P->N + 15) / 16) * (P->K / 128) + 1) : nullptr;
-  pv->ob = small ? c.take<uint32_t>((size_t)nnz + 4) : nullptr;
-  pv->ob_ptr = small ? c.take<int32_t>((size_t)((P->N + 127) / 128) * (P->K / 128) + 1) : nullptr;
+  pv->ob = blocks ? c.take<uint32_t>((size_t)nnz + 4) : nullptr;
+  pv->ob_ptr = blocks ? c.take<int32_t>((size_t)((P->N + 127) / 128) * (P->K / 128) + 1) : nullptr;
   // the scratch of the streaming path with transposed activations
   pv->xt = tiles ? c.take<char>(gwq_stream_scratch_bytes(P->K)) : nullptr;
 }
@@ -359,7 +359,6 @@ extern "C" gwq_status gwq_pack(const uint16_t* W, gwq_outliers* S, int32_t N, in
   P->N = N; P->K = K; P->bits = bits; P->group = group;
   P->S = nullptr; P->priv = pv;
   gwq_carver c = {nullptr, 0};
-  carve(c, P, pv, S->nnz);
   int dev = 0;
   verdict = static_cast<int32_t*>(gwq_pinned_slot());
   if (!verdict) {
@@ -368,6 +367,7 @@ extern "C" gwq_status gwq_pack(const uint16_t* W, gwq_outliers* S, int32_t N, in
   }
   GWQ_CUDA_TRY(cudaGetDevice(&dev));
   GWQ_CUDA_TRY(cudaDeviceGetAttribute(&pv->sm_count, cudaDevAttrMultiProcessorCount, dev));
+  carve(c, P, pv, S->nnz);
   GWQ_CUDA_TRY(gwq_dev_alloc(&base, c.used, stream));
   c = gwq_carver{static_cast<char*>(base), 0};
   carve(c, P, pv, S->nnz);

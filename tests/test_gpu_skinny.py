@@ -90,3 +90,34 @@ def test_give_up_path_of_the_streaming_kernel():
     assert gwq.gwq_device_status(P) == 0
     y_ref, bound = orc.linear(xv, w_hat)
     assert_linear_close(y, y_ref, bound)
+
+
+# Which kernel a layer beyond 5 M weights takes at 24 fp16 tokens, told by the workspace it asks for (two partial tiles per SM, or
+# the streaming kernel's copy of the activations, or the tensor-core kernel's nothing), and that its product is that
+# kernel's: fp16-rounded scaled weights would be 1.4e-4 off.
+@pytest.mark.parametrize("N,K,bits,group,taken", [
+    (2600, 2304, 3, 64, True),      # groups of 64 with 3 bits always
+    (2400, 6912, 4, 128, True),     # 150 tiles of 16 rows: two for the busiest SM, hardly more than one on average
+    (2400, 6912, 3, 128, True),
+    (2304, 6912, 4, 128, False),    # 144 tiles: one each
+    (2400, 2304, 4, 128, False),    # rows too short for the start-up to pay
+    (2400, 6912, 4, 64, False),
+    (2400, 6912, 2, 128, False),
+])
+def test_large_layers_take_the_kernel_that_the_rule_names(N, K, bits, group, taken):
+    W, G = synth.make_weight_and_grad(N, K, 130)
+    L = orc.quantize_layer(W, G, 0.02, bits, group)
+    P = quantize_on_gpu(W, G, 0.02, bits, group)
+    assert_packed_equal(P, L)
+    w_hat = oracle_w_hat(L)
+    partial_tiles = 2 * torch.cuda.get_device_properties(0).multi_processor_count * 32 * 128 * 4
+    for M in (17, 24, 32):
+        assert (gwq.load_library().gwq_linear_workspace_bytes(P._h, gwq.GWQ_F16, M) == partial_tiles) == taken
+        bits16, xv = synth.make_activations(M, K, seed=M, dtype="f16")
+        y_ref, bound = orc.linear(xv, w_hat)
+        y = gwq.gwq_linear(P, x_tensor(bits16, "f16"), out_dtype=torch.float32)
+        assert gwq.gwq_device_status(P) == 0
+        assert_linear_close(y, y_ref, bound)
+        err = y.double().cpu().numpy() - y_ref
+        assert np.sqrt(np.mean(err ** 2) / np.mean(y_ref ** 2)) < 3e-5
+    P.free()
