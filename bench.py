@@ -6,10 +6,11 @@ One "step" is one pass of gwq_linear over the Llama-7B-shaped decode layer set
 M = 1, 4 and 16 tokens: 42 products in 24 calls (sibling projections share a call),
 replayed as one CUDA graph.  The headline
 value is the HBM rate over the algorithmic bytes of that step.  Beside it the
-line reports per-layer decode times, the tensor-core prefill cases, the encode
-kernels, a dense fp16 GEMM (torch.matmul, a library call) on the unquantized
-weights, the end-to-end rate through the host-buffer entry point, and the CPU
-checker timed on the host cores.
+line on stdout reports the end-to-end rate through the host-buffer entry point,
+the best prefill case and the CPU checker timed on the host cores; tables of
+per-layer decode times, the tensor-core prefill cases, the encode kernels and a
+dense fp16 GEMM (torch.matmul, a library call) on the unquantized weights go to
+stderr.
 
   python bench.py --gpus 1 --steps 20 --warmup 3
   python bench.py --impl reference ...      (times the CPU checker instead)
@@ -882,6 +883,31 @@ def run_reference_arm(args):
             "gpu_launches": 0}
 
 
+# What the one line on stdout carries.  The tables beside the headline (some 30 KB) go to stderr, a line each, and to the file that
+# --tables names: whoever keeps only the end of the output still gets a whole line.
+TABLES = ("decode_cases", "llama70b_cases", "other_widths", "prefill", "decode_step_7b", "config0_single_layer", "cublas_fp16", "encode")
+
+
+def split_record(out: dict):
+    """(the record without its tables, the tables)."""
+    line = {k: v for k, v in out.items() if k not in TABLES}
+    tables = {k: out[k] for k in TABLES if k in out}
+    if "roofline" in line:
+        line["roofline"] = {k: v for k, v in line["roofline"].items() if not k.startswith("cases")}
+        tables.update({f"roofline_{k}": v for k, v in out["roofline"].items() if k.startswith("cases")})
+    return line, tables
+
+
+def print_record(out: dict, tables_file: str = "") -> None:
+    line, tables = split_record(out)
+    for name, table in tables.items():
+        print(json.dumps({name: table}, ensure_ascii=False), file=sys.stderr, flush=True)
+    if tables_file:
+        with open(tables_file, "w") as f:
+            json.dump(tables, f)
+    print(json.dumps(line, ensure_ascii=False), flush=True)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -897,6 +923,7 @@ def main():
     ap.add_argument("--skip-70b", action="store_true", help="skip the Llama-70B-shaped decode cases")
     ap.add_argument("--no-fuse", action="store_true",
                     help="launch sibling projections as separate concurrent calls instead of one gwq_linear_multi")
+    ap.add_argument("--tables", default="", metavar="FILE", help="write the tables beside the headline to FILE as well")
     ap.add_argument("--case", action="append", default=[], metavar="N,K,bits,group,M,dtype[,frac]",
                     help="time gwq_linear on one synthetic layer instead of the benchmark (repeatable)")
     ap.add_argument("--case-copies", type=int, default=0, help="packed copies cycled through (default: 256 MB worth)")
@@ -909,7 +936,7 @@ def main():
         return
     out = run_reference_arm(args) if args.impl == "reference" else run_cuda_arm(args)
     if out is not None:
-        print(json.dumps(out, ensure_ascii=False))
+        print_record(out, args.tables)
 
 
 if __name__ == "__main__":
