@@ -53,9 +53,10 @@ static __device__ __forceinline__ bool mbar_wait_warp(unsigned bar, unsigned par
 }
 
 // True while no kernel has given up on the layer (later calls then do no work until the host has read the status).  Other
-// CTAs write the word while this one starts, so a CTA must go by ONE read of it: one thread reads, before a barrier of all
-// that share its verdict, and hands it round through shared memory.  Warps that each looked for themselves could start with
-// different verdicts, and one that skips its loop never comes to the barriers inside it.
+// CTAs write the word while this one starts, so that two reads may differ.  Threads that meet at a warp-level operation or
+// at a barrier without a limit have to go by ONE read: of one lane, handed round the warp, or of one thread before a barrier of
+// all that share the verdict, handed round through shared memory.  (Warps that each looked for themselves could start
+// differently, and one that skips its loop never comes to a named barrier inside it.)
 static __device__ __forceinline__ bool no_one_gave_up(const int32_t* status) {
   return *reinterpret_cast<const volatile int32_t*>(status) == 0;
 }
