@@ -1,6 +1,6 @@
-// Host side of the decode path (M <= 32) of y = x (s (q - z) + S)^T (Section 3.2, Eq. "w"): choice of the
-// kernel variant, the token-major copy of the activations that the variants with more than 8 tokens gather
-// the outliers' activations from, and the launch.  The kernels are in decode_kernel.cuh.
+// Host side of the decode kernel with a CTA per tile of rows (decode_kernel.cuh; up to 32 tokens): choice of the variant, the
+// token-major copy of the activations that its ring variants gather the outliers' activations from, the launch, and the
+// rule that says which calls take it and which the streaming kernel (stream_kernel.cuh).
 #include "decode_kernel.cuh"
 
 namespace gwq_decode {
@@ -79,9 +79,9 @@ constexpr size_t kStageAllLimitTwoTiles = 96 * 1024;
 #define GWQ_TUNE_RT 0   // 1 / 2 force the tiles per CTA (tuning builds); 0: chosen from the grid size
 #endif
 
-// The variant for `count` layers that read the same x, or false when the streaming kernel has none: group size
-// 128 (M <= 32) or 64 (M <= 8; M <= 16 for layers up to kMaxWeights64Wide weights), K <= 65536 and a multiple of
-// 128, same K, group size and bit width in every layer, shared memory for at least a ring of two tiles.
+// The variant for `count` layers that read the same x, or false when this kernel has none: groups of 128 (M <= 32), of 64
+// (M <= 8; M <= 16 for layers up to kMaxWeights64Wide weights), of 32 (M <= 4) or of 16 (M = 1), K <= 65536 and a multiple
+// of 128, same K, group size and bit width in every layer, shared memory for at least a ring of two tiles.
 bool plan(const gwq_packed* const* P, int count, int M, Variant* v, int* cvcap) {
   if (count < 1 || count > kMaxLayers || M < 1 || M > 32) return false;
   const int group = P[0]->group;
@@ -199,7 +199,7 @@ bool gwq_decode_stages(const gwq_packed* const* P, int count, int M) {
   return plan(P, count, M, &v, &cvcap) && (v.nbuf == 0 || v.tp == 1);
 }
 
-// Decode launcher for `count` layers that read the same x.  Returns GWQ_ERR_UNSUPPORTED where the streaming kernel
+// Launcher for `count` layers that read the same x.  Returns GWQ_ERR_UNSUPPORTED where this kernel
 // has no variant (nothing has been launched then).  A token-major copy of x goes to `scratch`.
 gwq_status gwq_launch_decode_multi(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M,
                                    void* const* y, gwq_dtype yd, void* scratch, cudaStream_t stream) {

@@ -104,7 +104,8 @@ __device__ bool find_bin(const unsigned int* hist, unsigned int k, unsigned int*
   return found[0] != 0xFFFFFFFFu;
 }
 
-__device__ __forceinline__ unsigned int mix(unsigned int x) {   // spreads the sampled rows
+// Spreads the sampled rows: the 32-bit integer hash "lowbias32" of C. Wellons' hash-prospector (published, public domain).
+__device__ __forceinline__ unsigned int mix(unsigned int x) {
   x ^= x >> 16; x *= 0x7FEB352Du;
   x ^= x >> 15; x *= 0x846CA68Bu;
   return x ^ (x >> 16);
