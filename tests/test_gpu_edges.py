@@ -67,8 +67,8 @@ def test_one_group_per_row():
 @pytest.mark.parametrize("bits", [4, 3])
 def test_groups_of_64_on_the_streaming_path(bits):
     # a warp step of 128 columns holds two groups of 64, kept apart in two halves of the token block: wide rows whose
-    # activations are not staged up front (per-warp tiles), a partial last row block, up to 16 tokens (four token blocks
-    # beyond 8); with more tokens the tensor-core kernel takes over
+    # activations are not staged up front (per-warp tiles), a partial last row block; with 4 bits both decode kernels go on
+    # to 32 and 16 tokens, with 3 bits 17 fp16 tokens take the tcgen05 streaming kernel and 32 bf16 tokens the fused one
     _check(72, 8192, 0.01, bits, 64, 80 + bits, [(1, "f16"), (1, "bf16"), (3, "f16"), (5, "bf16"), (8, "f16"), (8, "bf16"),
                                                  (9, "f16"), (13, "bf16"), (16, "f16"), (16, "bf16"), (17, "f16"), (32, "bf16")])
     _check(40, 28672, 0.005, bits, 64, 84 + bits, [(1, "f16"), (4, "bf16"), (7, "f16"), (16, "bf16")])
@@ -80,16 +80,16 @@ def test_groups_of_64_with_an_odd_number_of_groups():
 
 
 def test_tall_layers_take_the_tensor_core_kernel_from_17_tokens():
-    # N >= 10240 with groups of 128: 17 to 32 tokens go to the tensor-core kernel's 32-token tile, fewer tokens
-    # and shorter layers stay on the streaming kernel; fused siblings follow the same rule
+    # many short rows with groups of 128 and 17 to 32 tokens: what decides between the tcgen05 streaming kernel (here the
+    # second layer with fp16 activations) and the mma.sync one is the layer, so that fused siblings follow the same rule
     _check(10368, 512, 0.01, 4, 128, 90, [(16, "f16"), (17, "f16"), (24, "bf16"), (32, "f16"), (32, "bf16")])
     _check(10240, 256, 0.01, 3, 128, 91, [(17, "bf16"), (32, "f16")])
 
 
 @pytest.mark.parametrize("bits", [4, 3])
 def test_two_tiles_per_cta(bits):
-    # 8192 rows: more 16-row blocks than one wave of CTAs, at most one wave of 32-row blocks, so up to 8 tokens the
-    # streaming kernel runs with two m16 tiles per CTA (staged activations here; a ragged last block: 8200 rows)
+    # 8192 rows: more 16-row blocks than one wave of CTAs, at most one wave of 32-row blocks, so up to 8 tokens the decode
+    # kernel with a CTA per tile runs with two m16 tiles per CTA where it takes the call (staged activations here; a ragged last block: 8200 rows)
     _check(8192, 256, 0.01, bits, 128, 92 + bits, [(1, "f16"), (1, "bf16"), (3, "f16"), (8, "f16"), (8, "bf16"), (16, "f16")])
     _check(8200, 128, 0.02, bits, 128, 96 + bits, [(1, "f16"), (5, "bf16")])
 

@@ -85,7 +85,7 @@ def test_tensor_core_path(layer, M, dtype):
     bits16, xv = synth.make_activations(M, P.K, seed=100 + M, dtype=dtype, heavy_channels=8)
     y_ref, bound = orc.linear(xv, w_hat)
     x = x_tensor(bits16, dtype)
-    y = gwq.gwq_linear(P, x, out_dtype=torch.float32)     # the binding's workspace: the two-phase path
+    y = gwq.gwq_linear(P, x, out_dtype=torch.float32)     # the binding's workspace: the two-phase path, or K in slices
     assert gwq.gwq_device_status(P) == 0
     assert_linear_close(y, y_ref, bound)
     # the fused kernel: a workspace without room for the expanded weights (none at all for fp16 activations)
@@ -199,7 +199,7 @@ def test_tensor_core_path_reads_back_columns_exactly_in_fp16():
 @pytest.mark.parametrize("layer", [(200, 1056, 0.01, 4, 16, 30), (200, 1056, 0.02, 3, 16, 31), (96, 1024, 0.01, 4, 32, 32)])
 @pytest.mark.parametrize("M,dtype", [(1, "f16"), (5, "bf16"), (16, "f16"), (40, "bf16"), (70, "f16")])
 def test_small_groups(layer, M, dtype):
-    # groups of 16 (the paper's own value, Section 3.2) and 32: the general kernel serves every M
+    # groups of 16 (the paper's own value, Section 3.2) and 32; K = 1056 is left to the general kernel for every M
     P, L, w_hat = _layer(*layer)
     bits16, xv = synth.make_activations(M, P.K, seed=60 + M, dtype=dtype)
     y_ref, bound = orc.linear(xv, w_hat)
@@ -220,7 +220,7 @@ SMALL_GROUP_LAYERS = [
                                      (33, "f16"), (300, "bf16"), (2100, "f16")])
 def test_small_groups_on_the_fast_paths(layer, M, dtype):
     # K a multiple of 128: groups of 16 and 32 run on the tensor cores (one scale per 16 or 32 columns inside the
-    # 64-column k-block; the weights expanded beforehand for many tokens) and, for one token, on the streaming kernel
+    # 64-column k-block; the weights expanded beforehand for many tokens) and, up to 32 mma columns, on the decode kernels
     P, L, w_hat = _layer(*layer)
     bits16, xv = synth.make_activations(M, P.K, seed=160 + M, dtype=dtype, heavy_channels=8 if M > 32 else 0)
     y_ref, bound = orc.linear(xv, w_hat)

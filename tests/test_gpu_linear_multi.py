@@ -55,7 +55,7 @@ def test_fused_siblings_match_checker_and_single_calls(bits, M, dtype):
 @pytest.mark.parametrize("bits", [4, 3])
 @pytest.mark.parametrize("M,dtype", [(1, "f16"), (4, "bf16"), (8, "f16"), (12, "f16")])
 def test_fused_siblings_with_groups_of_64(bits, M, dtype):
-    # one launch up to 8 tokens; beyond, one launch per layer on the tensor-core kernel
+    # one launch where the layers take one decode kernel by themselves, else one after the other
     sib = [_layer(N, 2176, 0.01, bits, 64, 50 + i) for i, N in enumerate((200, 72))]
     Ps = [s[0] for s in sib]
     bits16, xv = synth.make_activations(M, 2176, seed=200 + M, dtype=dtype)
@@ -68,7 +68,7 @@ def test_fused_siblings_with_groups_of_64(bits, M, dtype):
 
 
 def test_tall_siblings_beyond_16_tokens_follow_the_single_call():
-    # layers of 10240 rows or more go to the tensor-core kernel from 17 tokens on, in the fused call too
+    # from 17 tokens on small layers go to the tcgen05 streaming kernel, in the fused call too
     sib = [_layer(10240, 256, 0.01, 4, 128, 52), _layer(10368, 256, 0.01, 4, 128, 53)]
     for M in (16, 20):
         bits16, xv = synth.make_activations(M, 256, seed=210 + M, dtype="f16")

@@ -111,7 +111,7 @@ def test_tensor_core_paths(layer, M, dtype):
     bits16, xv = synth.make_activations(M, P.K, seed=100 + M, dtype=dtype, heavy_channels=8)
     y_ref, bound = orc.linear(xv, w_hat)
     x = x_tensor(bits16, dtype)
-    y = gwq.gwq_linear(P, x, out_dtype=torch.float32)     # the binding's workspace: the two-phase path
+    y = gwq.gwq_linear(P, x, out_dtype=torch.float32)     # the binding's workspace: the two-phase path, or K in slices
     assert gwq.gwq_device_status(P) == 0
     assert_linear_close(y, y_ref, bound)
     # the fused kernel: a workspace without room for the expanded weights (none at all for fp16 activations)
