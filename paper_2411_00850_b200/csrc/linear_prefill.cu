@@ -968,9 +968,9 @@ pair_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUt
       const long long t0 = clock64();
       while (clock64() - t0 < 200000) {}
     }
-    // MMAs that were issued may still read both CTAs' stages and write both tensor memories: one more commit arrives
-    // when all of them have completed; wait (bounded) for it before the pair leaves
-    if (warp == 1 && lane == 0 && rank == 0) {
+    // MMAs that were issued may still read both CTAs' stages and write both tensor memories: one more commit, of the lane that
+    // issued them, arrives when all of them have completed; wait (bounded) for it before the pair leaves
+    if (warp == 1 && rank == 0 && elect_one()) {
       int zero = 0;
       umma_commit_pair_local(drain_bar);
       (void)mbar_wait(drain_bar, 0, &zero, kSpinCycles);

@@ -88,7 +88,9 @@ static __device__ __forceinline__ uint64_t umma_desc(unsigned smem_addr) {
 
 // True in one lane of a converged warp.  MMAs are issued by that lane inside code that the whole warp runs, so that their
 // descriptors stay in uniform registers: from a branch that one thread takes, an MMA of up to 96 columns costs its issuer 54 cycles
-// and a chain of four 490; this way 16 at 32 columns with A in tensor memory, 40 with A in shared memory.
+// and a chain of four 490; this way 16 at 32 columns with A in tensor memory, 40 with A in shared memory.  The lane is the same one
+// every time (the election is deterministic for a mask) but need not be lane 0, and a tcgen05.commit tracks the MMAs of its own
+// thread alone: a kernel that issues by election also commits by election, on the give-up path too.
 static __device__ __forceinline__ bool elect_one() {
   unsigned elected;
   asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.b32 %0, 1, 0, p;\n}\n" : "=r"(elected));

@@ -48,3 +48,15 @@ def test_named_barriers_follow_a_verdict_of_all_their_warps(name):
 def test_every_wait_for_another_role_has_a_limit(name):
     text = _source(name)
     assert not re.search(r"mbarrier\.(try|test)_wait", text), "waits go through mbar_wait / mbar_wait_warp"
+
+
+@pytest.mark.parametrize("name", KERNELS)
+def test_mmas_and_their_commits_come_from_one_lane(name):
+    # a tcgen05.commit tracks the MMAs of the thread that makes it: from another lane it arrives at once, and what waits for it
+    # gives tensor memory and shared memory back under MMAs in flight
+    for text in _kernels(name):
+        lanes = set()
+        for call in re.finditer(r"\bumma_(?:f16|ts|commit)\w*\(", text):
+            conditions = re.findall(r"if \((?:[^\n]*\W)?(elected|elect_one\(\)|lane == 0)\W", text[:call.start()])
+            lanes.add("lane 0" if conditions[-1] == "lane == 0" else "elected")
+        assert len(lanes) == 1, "issued by one lane and committed by another"
