@@ -149,7 +149,8 @@ gwq_status gwq_pack(const uint16_t* W_f16, gwq_outliers* S, int32_t N, int32_t K
 
 /* Forward product y = x (s (q - z) + S)^T (Section 3.2, Eq. "w", outliers in FP16).
  *   x: device [M, K], fp16 or bf16 (x_dtype).  y: device [M, N], y_dtype one of
- *   F16 / BF16 / F32.  Accumulation is FP32.  M >= 1.  Up to 32 tokens take one of two bandwidth-bound decode
+ *   F16 / BF16 / F32.  Accumulation is FP32.  M >= 1.  A non-finite activation makes its token's results non-finite and no
+ *   other's.  Up to 32 tokens take one of two bandwidth-bound decode
  *   kernels (mma.sync) or, with a workspace, of large layers and of small groups a tcgen05 one, more tokens
  *   the tensor-core kernel (TMA, tcgen05, tensor memory).  With a workspace and more than 256 tokens (from 33 on where
  *   it is the faster way) that path expands the weights once instead of once per

@@ -18,11 +18,11 @@ AID_SRC = os.path.join(HERE, "bench_aid", "read_probe.cu")    # the benchmark's 
 AID_LIB = os.path.join(HERE, "bench_aid", "libbench_read_probe.so")
 EXT_SRC = os.path.join(CSRC, "torch_ext.cpp")
 EXT_LIB = os.path.join(HERE, "_gwq_torch.so")
-SOURCES = ("stream_w4_f16.cu", "stream_w4_bf16.cu", "stream_w3_f16.cu", "stream_w3_bf16.cu", "stream_w8_f16.cu",
+SOURCES = ("linear_skinny.cu", "stream_w4_f16.cu", "stream_w4_bf16.cu", "stream_w3_f16.cu", "stream_w3_bf16.cu", "stream_w8_f16.cu",
            "stream_w8_bf16.cu", "stream_w2_f16.cu", "stream_w2_bf16.cu",
            "decode_w4_f16.cu", "decode_w4_bf16.cu", "decode_w3_f16.cu", "decode_w3_bf16.cu", "decode_w8_f16.cu",
            "decode_w8_bf16.cu", "decode_w2_f16.cu", "decode_w2_bf16.cu", "alloc.cu", "select.cu",
-           "select_fast.cu", "select_static.cu", "pack.cu", "linear_simt.cu", "linear_decode.cu", "linear_stream.cu", "linear_skinny.cu", "linear_prefill.cu",
+           "select_fast.cu", "select_static.cu", "pack.cu", "linear_simt.cu", "linear_decode.cu", "linear_stream.cu", "linear_prefill.cu",
            "quality.cu", "gradmean.cu", "api.cu")
 NVCC_FLAGS = (
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",

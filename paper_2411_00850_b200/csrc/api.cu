@@ -192,11 +192,11 @@ static gwq_status linear_host(gwq_packed* P, const void* x_host, gwq_dtype xd, i
   const size_t xb = (size_t)M * P->K * dtype_bytes(xd), yb = (size_t)M * P->N * dtype_bytes(yd);
   gwq_status st = GWQ_OK;
   // Few tokens: what is pinned is read and written by the kernels themselves.  The activations are read once (by the
-  // transposing pre-pass, or, where every CTA reads them or looks for their largest, by a kernel that copies them first) and y is
+  // transposing pre-pass, or, where every CTA reads them, by a kernel that copies them first) and y is
   // written once, so that nothing is gained by the copy engine, whose two copies take longer than the product
   // (4096 x 11008 at 4 tokens: 47 -> 34 us).
   const bool skinny = wants_skinny(P, xd, M), direct = skinny || gwq_takes_decode(P, xd, M);
-  const bool copied = M == 1 || (skinny ? xd == GWQ_BF16 : direct && gwq_decode_ahead(P, xd, M));
+  const bool copied = M == 1 || (direct && !skinny && gwq_decode_ahead(P, xd, M));
   const void* x = direct && gwq_aligned16(x_host) ? device_view(x_host, xb) : nullptr;
   // (the kernels store element by element; the copy engine takes any address)
   const bool whole = (reinterpret_cast<uintptr_t>(y_host) & (dtype_bytes(yd) - 1)) == 0;

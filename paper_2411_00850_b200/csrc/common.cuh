@@ -87,7 +87,7 @@ bool gwq_decode_ahead(const gwq_packed* P, gwq_dtype xd, int M);   // the kernel
 gwq_status gwq_launch_prefill(const gwq_packed* P, const void* x, gwq_dtype xd, int M, void* y,
                               gwq_dtype yd, void* ws, size_t ws_bytes, cudaStream_t stream);
 size_t gwq_prefill_workspace_bytes(const gwq_packed* P, gwq_dtype xd, int M);
-bool gwq_skinny_takes(const gwq_packed* P, int M);   // the tcgen05 decode kernel has a variant for (P, M)
+bool gwq_skinny_takes(const gwq_packed* P, gwq_dtype xd, int M);   // the tcgen05 decode kernel has a variant for (P, xd, M)
 bool gwq_skinny_ahead(const gwq_packed* P, gwq_dtype xd, int M);   // ... and is the fastest one
 bool gwq_skinny_before(const gwq_packed* P, gwq_dtype xd, int M);  // ... and has always served the call
 size_t gwq_skinny_workspace_bytes(const gwq_packed* const* P, int count, gwq_dtype xd, int M);

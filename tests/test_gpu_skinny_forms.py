@@ -53,6 +53,35 @@ def test_forms(N, K, frac, bits, group, crowd, calls):
     P.free()
 
 
+# bf16 activations are multiplied as they are: a channel 2^70 above the others leaves the rest of a row's sum alone where its weight
+# is zero, a common power of two comes out again exactly, and one infinite activation spoils its own token only (fp16 too).
+@pytest.mark.parametrize("N,K,frac,bits,group,M", [(300, 1152, 0.01, 3, 16, 8), (260, 640, 0.02, 4, 32, 16), (137, 2176, 0.05, 2, 32, 17),
+                                                   (1500, 1920, 0.01, 3, 64, 32)])
+def test_range_of_activations(N, K, frac, bits, group, M):
+    W, G = synth.make_weight_and_grad(N, K, N + K)
+    far, G[:, K // 2 + 3] = K // 2 + 3, 0.0
+    W[::2, far] = 0.0
+    P, w_hat = quantize_on_gpu(W, G, frac, bits, group), oracle_w_hat(orc.quantize_layer(W, G, frac, bits, group))
+    bits16, xv = synth.make_activations(M, K, seed=M, dtype="bf16", heavy_channels=8)
+    x = x_tensor(bits16, "bf16")
+    y = gwq.gwq_linear(P, x, out_dtype=torch.float32)
+    for power in (2.0 ** 112, 2.0 ** -80):
+        assert torch.equal(gwq.gwq_linear(P, x * power, out_dtype=torch.float32), y * power)
+    x[:, far], xv[:, far] = 2.0 ** 70, 2.0 ** 70
+    y_ref, bound = orc.linear(xv, w_hat)
+    err = np.abs(gwq.gwq_linear(P, x, out_dtype=torch.float32).double().cpu().numpy() - y_ref)
+    assert np.all(err <= (K + 72) * 2.0 ** -23 * bound + 1e-30), float((err / bound).max())
+    for dtype in ("f16", "bf16"):
+        x = x_tensor(synth.make_activations(M, K, seed=M, dtype=dtype)[0], dtype)
+        y = gwq.gwq_linear(P, x)
+        x[M - 2, far] = float("inf")
+        spoilt = gwq.gwq_linear(P, x)
+        assert not bool(torch.isfinite(spoilt[M - 2]).any())
+        assert torch.equal(torch.cat((spoilt[:M - 2], spoilt[M - 1:])), torch.cat((y[:M - 2], y[M - 1:])))
+    assert gwq.gwq_device_status(P) == 0
+    P.free()
+
+
 def test_layers_of_one_call_give_the_bits_of_the_single_calls():
     layers = [_layer(N, 1152, 0.02, 4, 16)[0] for N in (260, 5, 3000)]
     for M, dtype in ((8, "f16"), (13, "bf16")):
@@ -61,7 +90,7 @@ def test_layers_of_one_call_give_the_bits_of_the_single_calls():
             assert torch.equal(many, gwq.gwq_linear(P, x))
 
 
-# Host buffers: fp16 activations are read by the pre-pass where they are, bf16 ones are copied first.
+# Host buffers: activations are read by the pre-pass where they are.
 @pytest.mark.parametrize("M,dtype", [(7, "f16"), (20, "bf16")])
 def test_host_buffers(M, dtype):
     P, _ = _layer(300, 1152, 0.02, 3, 16 if M <= 16 else 64)
