@@ -1345,20 +1345,28 @@ __global__ void __launch_bounds__(256) expand_block_kernel(const uint32_t* __res
 // When the weights are expanded once instead of once per token tile.  The expansion is a pass of 2.5 bytes per weight
 // (24 us for 45 M weights, 125 us for 235 M); the contraction on CTA pairs then runs at 1000 to 1500 TFLOP/s, where the
 // fused kernel is bound by its dequantisation warps and expands the weights again for every token tile of 256.  So: more than
-// 256 tokens always; up to there by two measured costs, in us: the fused kernel 3 + 0.1 per token + 0.49 per k-block and round of its
-// 128-row tiles over the SMs, the two-phase path 0.94 (33 tokens) to 1.08 (256) per million weights.  Within 4 % of both on
-// 11008 x 4096, 10240 x 10240, 13824 x 5120, 14336 x 4096, 18000 x 4096 and 9600 x 8192 at 33 to 256 tokens.  Two-phase / fused there: at
-// 33 tokens 43.3 / 38.5, 102 / 82, 66 / 47, 54 / 39, 65 / 40, 78 / 68; at 128 45.4 / 47.4, 104 / 92, 68 / 56, 55.5 / 47.8, 68 / 49, 80 / 77; at 256
-// 54.7 / 61.6, 115 / 112, 75 / 71, 62 / 62, 74 / 64, 88 / 95.  (Two rounds of tiles: 28672 x 8192 at 128 tokens 237 / 141.)
+// 256 tokens always; up to there by two costs in us.  The fused kernel: a start, the tokens' stores, and a k-block after the other in
+// every round of its 128-row tiles over the SMs, longer with wider codes, with more scales per k-block (whose token tile is always 256)
+// and with larger token tiles.  The two-phase path: a start, the expansion by weights and width, the contraction by k-blocks.  Fitted to
+// 3040 calls (19 layers of 2048 x 256 to 9600 x 16384 whose tiles leave no room for slices, every width and group size, 33 to 256 tokens)
+// with a deviation of 5 %.  Where they are close, layers of one round take the two-phase path and wider ones the fused kernel: those
+// are the ones that always did.  Two-phase / fused, 4 bits in groups of 128: 18000 x 4096 at 33 tokens 71 / 40, 10240 x 10240 at 33 108 / 82,
+// 11008 x 4096 at 129 57 / 52; 8 bits in groups of 32: 9600 x 8192 at 128 95 / 107; 16000 x 1024, groups of 32, bf16, at 33 20.5 / 24.9.
 constexpr int kExpandAlwaysTokens = 257;   // more than one token tile of the fused kernel
-static bool wants_expansion(const gwq_packed* P, int M) {
+static bool wants_expansion(const gwq_packed* P, gwq_dtype xd, int M) {
 #ifdef GWQ_TUNE_EXPAND_MIN
   return M >= GWQ_TUNE_EXPAND_MIN;
 #endif
   if (M <= 32 || M >= kExpandAlwaysTokens) return M > 32;
   const gwq_priv* pv = static_cast<const gwq_priv*>(P->priv);
   const int sms = pv->sm_count > 0 ? pv->sm_count : 148, tiles = (P->N + kTileN - 1) / kTileN, rounds = (tiles + sms - 1) / sms;
-  return (0.94 + 0.00055 * M) * 1e-6 * ((double)P->N * P->K) < 3.0 + 0.1 * M + 0.49 * (P->K / kBlockK) * rounds;
+  const bool bf = xd == GWQ_BF16, small = P->group < 64;
+  const double kb = P->K / kBlockK, weights = 1e-6 * P->N * P->K;
+  const double step = (P->bits == 8 ? 0.61 : P->bits == 3 ? 0.48 : 0.45) + (small ? 0.10 : M > 128 ? 0.09 : M > 64 ? 0.03 : 0.0);
+  const double fused = 6.3 + (bf ? 3.8 : 0.0) + (small ? 3.0 : 0.0) + 0.08 * M + step * kb * rounds;
+  const double two = 7.2 + (bf ? 2.0 + 2.9e-6 * M * P->K : 0.0) + (P->bits == 8 ? 0.72 : P->bits == 3 ? 0.65 : 0.59) * weights +
+                     (M > 128 ? 0.30 : 0.22) * kb + 0.71e-6 * P->N * M;
+  return two < fused * (rounds > 1 ? 0.96 : 1.04);
 }
 // One tile of tokens (33 to 256) whose tiles of features leave half of the SMs idle or more: the fused kernel with K in
 // slices.  It was the two-phase path's before (3669 x 11008, 77 tokens: 45 -> 30 us, 256: 51 -> 38; 8192 x 8192 bf16, 33
@@ -1411,7 +1419,7 @@ size_t gwq_prefill_workspace_bytes(const gwq_packed* P, gwq_dtype xd, int M) {
   // (the expanded weights are followed by the FP32 partial tiles of the K-slices)
   return x16_bytes(P, xd, M) +
          (wants_slices(P, M)      ? slice_sum_bytes(P, M)
-          : wants_expansion(P, M) ? (((size_t)P->N * P->K * 2 + 255) & ~(size_t)255) + pair_partial_bytes(pv->sm_count)
+          : wants_expansion(P, xd, M) ? (((size_t)P->N * P->K * 2 + 255) & ~(size_t)255) + pair_partial_bytes(pv->sm_count)
                                   : 0);
 }
 
@@ -1439,7 +1447,7 @@ gwq_status gwq_launch_prefill(const gwq_packed* P, const void* x, gwq_dtype xd, 
   float* sums = nullptr;
   if (wants_slices(P, M) && ws && ws_bytes >= gwq_prefill_workspace_bytes(P, xd, M)) {
     sums = reinterpret_cast<float*>(static_cast<char*>(ws) + xb);
-  } else if (wants_expansion(P, M) && ws && ws_bytes >= gwq_prefill_workspace_bytes(P, xd, M)) {
+  } else if (wants_expansion(P, xd, M) && ws && ws_bytes >= gwq_prefill_workspace_bytes(P, xd, M)) {
     char* w16 = static_cast<char*>(ws) + xb;
     float* partial = reinterpret_cast<float*>(w16 + (((size_t)P->N * P->K * 2 + 255) & ~(size_t)255));
     const gwq_status st = launch_expanded(P, x, tok_scale, reinterpret_cast<uint16_t*>(w16), partial, M, y, yd, stream);

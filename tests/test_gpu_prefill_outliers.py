@@ -34,3 +34,17 @@ def test_outliers_of_prompts(N, K, frac, bits, group):
     bits16, xv = synth.unit_activations(cols, K, "f16")
     assert_linear_close(gwq.gwq_linear(P, x_tensor(bits16, "f16"), out_dtype=torch.float32), *orc.linear(xv, w_hat))
     P.free()
+
+
+# Which path a prompt takes, told by the workspace it asks for: the expanded weights, or not.  Both sides of the line measured (us,
+# two-phase / fused): 20.5 / 24.9, 98 / 112, 71 / 40, 57 / 52, 76 / 47.
+@pytest.mark.parametrize("N,K,bits,group,dtype,M,expanded", [
+    (16000, 1024, 4, 32, "bf16", 33, True), (9600, 8192, 8, 32, "bf16", 128, True), (18000, 4096, 4, 128, "f16", 33, False),
+    (11008, 4096, 4, 128, "f16", 129, False), (18000, 4096, 8, 128, "f16", 33, False),
+])
+def test_choice_of_the_prompt_path(N, K, bits, group, dtype, M, expanded):
+    W = torch.full((N, K), 0.5, dtype=torch.float16, device="cuda")
+    P = gwq.gwq_pack(W, gwq.gwq_select_outliers(W, torch.zeros(N, K, device="cuda"), 0.0), bits, group)
+    xd = gwq.GWQ_F16 if dtype == "f16" else gwq.GWQ_BF16
+    assert (gwq.load_library().gwq_linear_workspace_bytes(P._h, xd, M) >= 2 * N * K) == expanded
+    P.free()
