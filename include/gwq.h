@@ -185,8 +185,8 @@ gwq_status gwq_linear_ws(const gwq_packed* P, const void* x, gwq_dtype x_dtype, 
  *   x: device [M, K]; y: host array of `count` device pointers, y[i] is [M, P[i]->N], all of y_dtype.
  *   With M <= 32, one group size and one bit width for all layers, the products run as ONE kernel launch wherever
  *   all layers take the same decode kernel by themselves (with 9 to 32 tokens layer 0 lends its scratch: do not overlap
- *   with another such call that uses P[0]); otherwise the call is the same as `count` calls of gwq_linear in order
- *   (and like them returns GWQ_ERR_WORKSPACE where a product needs scratch).  Asynchronous on `stream`; never
+ *   with another such call that uses P[0]), with a workspace also those layers that do where not all of them do; otherwise the call
+ *   is the same as `count` calls of gwq_linear (and like them returns GWQ_ERR_WORKSPACE where a product needs scratch).  Asynchronous on `stream`; never
  *   allocates, never synchronises.
  * gwq_linear_multi_ws: with scratch memory supplied by the caller, as in gwq_linear_ws (each product is then exactly the one
  *   gwq_linear_ws computes); gwq_linear_multi_workspace_bytes: its size.

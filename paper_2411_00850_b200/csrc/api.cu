@@ -96,11 +96,25 @@ extern "C" gwq_status gwq_linear(const gwq_packed* P, const void* x, gwq_dtype x
   return gwq_linear_ws(P, x, xd, M, y, yd, nullptr, 0, stream_);
 }
 
-// Several layers of up to 32 tokens as one launch: the tcgen05 decode kernel takes each of them by itself (1), or none (0).
-static int launches_as_one(const gwq_packed* const* P, int count, gwq_dtype xd, int M) {
-  int skinny = 0;
-  for (int i = 0; i < count; ++i) skinny += wants_skinny(P[i], xd, M) && P[i]->bits == P[0]->bits && P[i]->group == P[0]->group;
-  return M > GWQ_DECODE_MAX_M || (skinny > 0 && skinny < count) ? -1 : skinny > 0;
+// The layers of a call of up to 32 tokens that the tcgen05 decode kernel takes by themselves, or the others: each kind goes as one
+// launch (one by one about 64 us, so 53 on 8192 + 4096 + 4096 rows x 8192 in groups of 64 at 16 tokens, where the first is of the one kind;
+// 51 and 36 on 4096 + 1024 + 1024 rows x 4096 at 32).
+struct Kind {
+  const gwq_packed* P[GWQ_MULTI_MAX];
+  void* y[GWQ_MULTI_MAX];
+  int count;
+  bool alike;   // one width and one group size
+};
+static Kind layers_of_kind(bool skinny, const gwq_packed* const* P, void* const* y, int count, gwq_dtype xd, int M) {
+  Kind k = {};
+  k.alike = true;
+  for (int i = 0; i < count; ++i) {
+    if (wants_skinny(P[i], xd, M) != skinny) continue;
+    k.P[k.count] = P[i];
+    k.y[k.count++] = y ? y[i] : nullptr;
+    k.alike = k.alike && P[i]->bits == k.P[0]->bits && P[i]->group == k.P[0]->group;
+  }
+  return k;
 }
 
 static bool valid_layers(const gwq_packed* const* P, int32_t count, int32_t M) {
@@ -112,13 +126,39 @@ static bool valid_layers(const gwq_packed* const* P, int32_t count, int32_t M) {
 
 extern "C" size_t gwq_linear_multi_workspace_bytes(const gwq_packed* const* P, int32_t count, gwq_dtype xd, int32_t M) {
   if (!valid_layers(P, count, M) || (xd != GWQ_F16 && xd != GWQ_BF16)) return 0;
-  const int one = launches_as_one(P, count, xd, M);
-  size_t need = one == 1 ? gwq_skinny_workspace_bytes(P, count, xd, M) : one == 0 ? few_scratch(P, count, xd, M) : 0;
+  size_t need = 0;
+  if (M <= GWQ_DECODE_MAX_M) {
+    const Kind few = layers_of_kind(false, P, nullptr, count, xd, M), skinny = layers_of_kind(true, P, nullptr, count, xd, M);
+    if (few.count > 0) need = few_scratch(few.P, few.count, xd, M);
+    const size_t wide = skinny.count > 0 && skinny.alike ? gwq_skinny_workspace_bytes(skinny.P, skinny.count, xd, M) : 0;
+    need = wide > need ? wide : need;
+  }
   for (int i = 0; i < count; ++i) {
     const size_t own = gwq_linear_workspace_bytes(P[i], xd, M);
     need = own > need ? own : need;
   }
   return need;
+}
+
+static gwq_status one_by_one(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M, void* const* y, gwq_dtype yd,
+                             void* ws, size_t ws_bytes, cudaStream_t stream) {
+  for (int i = 0; i < count; ++i) {
+    const gwq_status st = gwq_linear_ws(P[i], x, xd, M, y[i], yd, ws, ws_bytes, stream);
+    if (st != GWQ_OK) return st;
+  }
+  return GWQ_OK;
+}
+// Layers that are not the tcgen05 kernel's (or a call without a workspace): one launch where they share a kernel.
+static gwq_status few_together(const gwq_packed* const* P, int count, const void* x, gwq_dtype xd, int M, void* const* y, gwq_dtype yd,
+                                void* ws, size_t ws_bytes, cudaStream_t stream) {
+  const size_t need = few_scratch(P, count, xd, M);
+  void* scratch = scratch_in(ws, ws_bytes, need);
+  if (!scratch && M > kMostTokensAlone) scratch = own_scratch(P[0]);
+  if (scratch || need == 0) {
+    const gwq_status st = launch_few(P, count, x, xd, M, y, yd, scratch, stream);
+    if (st != GWQ_ERR_UNSUPPORTED) return st;
+  }
+  return one_by_one(P, count, x, xd, M, y, yd, ws, ws_bytes, stream);
 }
 
 extern "C" gwq_status gwq_linear_multi_ws(const gwq_packed* const* P, int32_t count, const void* x, gwq_dtype xd, int32_t M,
@@ -130,23 +170,18 @@ extern "C" gwq_status gwq_linear_multi_ws(const gwq_packed* const* P, int32_t co
   for (int i = 0; i < count; ++i)
     if (!y[i] || !gwq_aligned16(y[i])) return GWQ_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-  const int one = launches_as_one(P, count, xd, M);
-  if (one == 1 && ws && aligned256(ws) && ws_bytes >= gwq_skinny_workspace_bytes(P, count, xd, M))
-    return gwq_launch_skinny(P, count, x, xd, M, y, yd, ws, stream);
-  if (M <= GWQ_DECODE_MAX_M && (!ws || one == 0)) {
-    const size_t need = few_scratch(P, count, xd, M);
-    void* scratch = scratch_in(ws, ws_bytes, need);
-    if (!scratch && M > kMostTokensAlone) scratch = own_scratch(P[0]);
-    if (scratch || need == 0) {
-      const gwq_status st = launch_few(P, count, x, xd, M, y, yd, scratch, stream);
-      if (st != GWQ_ERR_UNSUPPORTED) return st;
+  if (M <= GWQ_DECODE_MAX_M && !ws) return few_together(P, count, x, xd, M, y, yd, nullptr, 0, stream);
+  if (M <= GWQ_DECODE_MAX_M) {
+    const Kind few = layers_of_kind(false, P, y, count, xd, M), skinny = layers_of_kind(true, P, y, count, xd, M);
+    if (few.count > 0) {
+      const gwq_status st = few_together(few.P, few.count, x, xd, M, few.y, yd, ws, ws_bytes, stream);
+      if (st != GWQ_OK) return st;
     }
+    if (skinny.count > 0 && skinny.alike && aligned256(ws) && ws_bytes >= gwq_skinny_workspace_bytes(skinny.P, skinny.count, xd, M))
+      return gwq_launch_skinny(skinny.P, skinny.count, x, xd, M, skinny.y, yd, ws, stream);
+    return one_by_one(skinny.P, skinny.count, x, xd, M, skinny.y, yd, ws, ws_bytes, stream);
   }
-  for (int i = 0; i < count; ++i) {   // more tokens than the streaming kernel takes, or layers of different kinds
-    const gwq_status st = gwq_linear_ws(P[i], x, xd, M, y[i], yd, ws, ws_bytes, stream_);
-    if (st != GWQ_OK) return st;
-  }
-  return GWQ_OK;
+  return one_by_one(P, count, x, xd, M, y, yd, ws, ws_bytes, stream);
 }
 
 extern "C" gwq_status gwq_linear_multi(const gwq_packed* const* P, int32_t count, const void* x, gwq_dtype xd,

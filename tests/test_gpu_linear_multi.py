@@ -81,6 +81,39 @@ def test_tall_siblings_beyond_16_tokens_follow_the_single_call():
             assert gwq.gwq_device_status(P) == 0
 
 
+def _launches(call):
+    """Kernels that `call` enqueues."""
+    graph, n = torch.cuda.CUDAGraph(keep_graph=True), C.c_size_t()
+    with torch.cuda.graph(graph):
+        call()
+    assert C.CDLL("libcudart.so.12").cudaGraphGetNodes(C.c_void_p(graph.raw_cuda_graph()), None, C.byref(n)) == 0
+    return n.value
+
+
+def test_siblings_that_take_different_kernels_go_kind_by_kind():
+    # 20 fp16 tokens: layers of up to 5 M weights take the tcgen05 decode kernel (three launches), larger ones of short rows another
+    # (a pre-pass and the product); the layers of a kind share theirs whatever their order
+    shapes = ((1000, 1024), (5376, 1024), (200, 1024), (5500, 1024))
+    Ps = []
+    for i, (N, K) in enumerate(shapes):
+        W, G = synth.make_weight_and_grad(N, K, 70 + i)
+        Ps.append(quantize_on_gpu(W, G, 0.01, 4, 128))
+    x = x_tensor(synth.make_activations(20, 1024, seed=70, dtype="f16")[0], "f16")
+    single = [gwq.gwq_linear(P, x) for P in Ps]
+    for order in ((0, 1, 2, 3), (1, 0, 3), (3, 2)):
+        for i, y in zip(order, gwq.gwq_linear_multi([Ps[i] for i in order], x)):
+            assert torch.equal(y, single[i])
+    outs = [torch.empty_like(y) for y in single]
+    assert [_launches(lambda: gwq.gwq_linear(P, x, out=y)) for P, y in zip(Ps, outs)] == [3, 2, 3, 2]
+    assert _launches(lambda: gwq.gwq_linear_multi(Ps, x, outs=outs)) == 5
+    mixed = quantize_on_gpu(*synth.make_weight_and_grad(300, 1024, 75), 0.01, 3, 64)   # of the first kind, another form
+    for y, P in zip(gwq.gwq_linear_multi([mixed, Ps[0], Ps[1]], x), (mixed, Ps[0], Ps[1])):
+        assert torch.equal(y, gwq.gwq_linear(P, x))
+    for P in Ps + [mixed]:
+        assert gwq.gwq_device_status(P) == 0
+        P.free()
+
+
 def test_two_and_four_layers_and_16_bit_outputs():
     sib = _siblings(4) + [_layer(48, 1024, 0.02, 4, 128, 47)]
     bits16, xv = synth.make_activations(4, 1024, seed=7, dtype="f16")
