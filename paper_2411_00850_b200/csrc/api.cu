@@ -3,7 +3,7 @@
 #include "common.cuh"
 
 #ifndef GWQ_DECODE_MAX_M
-#define GWQ_DECODE_MAX_M 32   // up to here the streaming kernel; above, the tcgen05 kernels
+#define GWQ_DECODE_MAX_M 32   // up to here the decode kernels; above, the kernels of prompts
 #endif
 
 static size_t dtype_bytes(gwq_dtype d) { return d == GWQ_F32 ? 4 : 2; }

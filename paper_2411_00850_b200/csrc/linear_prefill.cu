@@ -804,7 +804,7 @@ pair_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUt
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issue (first CTA of the pair)
-    // By the whole warp and an elected lane (elect_one): 28672 x 8192 at 2048 tokens 764 -> 738 us, 4096 x 4096 at 384 31.7 ->
+    // By the whole warp and an elected lane (elect_one): 28672 x 8192 at 2048 tokens 764 -> 738 us while the power cap does not hold (else level), 4096 x 4096 at 384 31.7 ->
     // 29.2, 11008 x 4096 at 256 61.6 -> 59.5.  (The fused kernel, whose dequantising warps need the issue slots, is 7 to 10 % slower that way.)
     if (rank == 0) {
       // instruction descriptor: FP32 accumulate, A and B fp16, K-major, N = 256, M = 256 (128 rows per CTA)
