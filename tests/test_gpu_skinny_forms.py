@@ -150,7 +150,7 @@ def test_large_layers(N, K, bits, group, M, dtype):
     P.free()
 
 
-# Which kernel a call takes, told by the workspace it asks for (partial sums, or the other kernels' copy of the activations at most), on
+# Which kernel a call takes, told by the workspace it asks for (partial sums, or the other kernels' copy of the activations or nothing), on
 # both sides of the lines (us, the others' / this kernel's): 14.8 / 16.6, 18.9 / 14.7, 22.2 / 24.4, 27.6 / 25.7, 57.5 / 63.4, 68.7 / 63.3,
 # 19.2 / 20.9, 30.8 / 35.2, 35.2 / 33.5; 8-bit codes with bf16 activations have no variant.
 @pytest.mark.parametrize("N,K,bits,group,dtype,M,taken", [
@@ -163,5 +163,5 @@ def test_choice_of_the_decode_kernel(N, K, bits, group, dtype, M, taken):
     W = torch.full((N, K), 0.5, dtype=torch.float16, device="cuda")
     P = gwq.gwq_pack(W, gwq.gwq_select_outliers(W, torch.zeros(N, K, device="cuda"), 0.0), bits, group)
     asked = gwq.load_library().gwq_linear_workspace_bytes(P._h, gwq.GWQ_F16 if dtype == "f16" else gwq.GWQ_BF16, M)
-    assert (asked > K // 128 * 8576) == taken
+    assert (asked not in (0, K // 128 * 8576)) == taken
     P.free()
